@@ -643,10 +643,13 @@ cow_status cow_mse_grad(const float *rgb, const float *target, int64_t n, float 
  *     (measured 4 % faster at 1080p); used when the call's views select at
  *     most 96 block records in total, otherwise the call runs as
  *     COW_SCHED_THREAD;
- *   COW_SCHED_WARP: one ray per warp, the 32 lanes on 32 consecutive lattice
- *     samples of that ray, the in-block weights of Eq. 1 as a prefix product
- *     across the lanes (measured slower on aerial views: rays of one tile are
- *     marched one after another, so their texels are fetched again).
+ *     a call of at most 77824 pixels (those that fill the chip at one ray per
+ *     thread) marches one ray per warp instead, the 32 lanes on the ray's next
+ *     32 occupied samples, composited in order (the same image);
+ *   COW_SCHED_WARP: one ray per warp for frames of any size, each warp taking
+ *     32 rays of its tile one after another, records in shared memory (measured
+ *     slower on large aerial views: rays of one tile are marched one after
+ *     another, so their texels are fetched again).
  * Errors: INVALID_ARG for a null context or an unknown schedule. */
 #define COW_SCHED_WARP 0
 #define COW_SCHED_THREAD 1
@@ -659,11 +662,11 @@ cow_status cow_set_schedule(cow_ctx *ctx, int32_t schedule);
  * batch of at least 8192 rays is marched in a coherent order -- rays grouped
  * by the cell of their entry into the call's blocks' bounding box (8 x 8 x 8)
  * and of their direction (8 x 8 x 8), by a counting sort on the device -- so
- * that the rays of one warp gather neighbouring texels; random training rays
- * otherwise send every lane of a warp to a different line (measured on 2^20
- * random rays over 2x2 blocks of 128^3 / 512^2 FP32 features: forward 75.8
- * -> 44.3 ms, backward 170 -> 135 ms).  COW_RAY_ORDER_GIVEN: thread t marches
- * ray t.  Outputs are written at each ray's own index either way and each
+ * that the rays on the chip at one time gather neighbouring texels and share
+ * them in L2 (measured on 2^20 random rays over 2x2 blocks of 128^3 / 512^2
+ * FP32 features: forward 39.9 -> 31.1 ms).  COW_RAY_ORDER_GIVEN: warp t marches
+ * ray t.  cow_render_rays of 2^17 rays or more that are mostly alike their
+ * neighbours (a camera's rays) are marched one ray per thread in the given order.  Outputs are written at each ray's own index either way and each
  * ray's values are the same; gradient sums change only by the order of their
  * FP32 reductions.  The order costs a key pass, a scan and a scatter (about
  * 12 bytes a ray and 1 MiB of context scratch).  Errors: INVALID_ARG. */

@@ -558,9 +558,12 @@ void make_ray_recs(const cow_ctx *c, const int32_t *ids, int32_t n, cow::RayRecs
 constexpr int64_t kRayOrderMin = 8192;
 
 cow_status ray_order(cow_ctx *c, const float *o, const float *d, int64_t n, const int32_t *ids, int32_t n_ids,
-                     cudaStream_t st, const int32_t **perm) {
+                     cudaStream_t st, const int32_t **perm, const uint32_t **alike = nullptr) {
     *perm = nullptr;
-    if (c->ray_order != COW_RAY_ORDER_COHERENT || n < kRayOrderMin || n > 0x7fffffff) return COW_OK;
+    if (alike) *alike = nullptr;
+    const bool sort = c->ray_order == COW_RAY_ORDER_COHERENT && n >= kRayOrderMin;
+    const bool count = alike && n >= cow::kRaysAlikeMin;
+    if (!(sort || count) || n > 0x7fffffff) return COW_OK;
     float lo[3] = {3.0e38f, 3.0e38f, 3.0e38f}, hi[3] = {-3.0e38f, -3.0e38f, -3.0e38f};
     for (int32_t k = 0; k < n_ids; k++) {
         const BlockHost &b = c->blocks[(size_t)ids[k]];
@@ -571,10 +574,11 @@ cow_status ray_order(cow_ctx *c, const float *o, const float *d, int64_t n, cons
     }
     COW_CUDA(c->ray_keys.reserve((size_t)n * sizeof(uint32_t)));
     COW_CUDA(c->ray_hist.reserve((size_t)cow::kRayOrderHistWords * sizeof(uint32_t)));
-    COW_CUDA(c->ray_perm.reserve((size_t)n * sizeof(int32_t)));
+    if (sort) COW_CUDA(c->ray_perm.reserve((size_t)n * sizeof(int32_t)));
     COW_CUDA(cow::launch_ray_order(o, d, n, lo, hi, (uint32_t *)c->ray_keys.p, (uint32_t *)c->ray_hist.p,
-                                   (int32_t *)c->ray_perm.p, st));
-    *perm = (const int32_t *)c->ray_perm.p;
+                                   sort ? (int32_t *)c->ray_perm.p : nullptr, st));
+    if (sort) *perm = (const int32_t *)c->ray_perm.p;
+    if (count) *alike = (const uint32_t *)c->ray_hist.p + cow::kRayOrderAlike;
     return COW_OK;
 }
 
@@ -987,6 +991,7 @@ cow_status cow_render(cow_ctx *ctx, const cow_camera *cams, int32_t n_views, con
     a.err = ctx->d_err;
     a.test_flags = ctx->test_flags;
     a.wait_polls = ctx->wait_polls;
+    a.n_rays = plan.n_pix;
     if (block_mlp) {
         a.block_mlps = (const float *const *)((unsigned char *)ctx->views.p + vbytes + rbytes);
         a.n_freq = ctx->n_freq;
@@ -1072,7 +1077,9 @@ static cow_status render_rays_impl(cow_ctx *ctx, const float *o, const float *d,
         a.block_mlp_stride = ctx->block_mlp_nparam;
         a.n_freq = ctx->n_freq;
     }
-    if ((rc = ray_order(ctx, o, d, n_rays, ids, n_ids, st, &a.ray_perm)) != COW_OK) return rc;
+    if ((rc = ray_order(ctx, o, d, n_rays, ids, n_ids, st, &a.ray_perm,
+                        out_block_T || out_block_state ? nullptr : &a.ray_alike)) != COW_OK)
+        return rc;
     cow::RayRecs rr;
     make_ray_recs(ctx, ids, n_ids, rr);
     COW_CUDA(cow::launch_march_rays(a, rr, st));

@@ -25,7 +25,7 @@ struct MarchArgs {
     unsigned *err;
     const float *ray_o;    // ray mode
     const float *ray_d;
-    int64_t n_rays;
+    int64_t n_rays;        // rays of the call (view mode: pixels)
     int32_t smem_recs;     // view mode, thread schedule: block records the launch's shared memory holds
     const float *const *block_mlps;  // view mode, per-block MLPs: weights of record k, parallel to recs
     int32_t n_freq;                  // PE frequencies of the per-block MLPs
@@ -36,7 +36,8 @@ struct MarchArgs {
     uint32_t wait_polls;             // bound on each mbarrier wait (0: the kernel's default)
     float *out_partials;             // block-parallel form: n_rays x n_ids x 8 per-block partials (written)
     const float *in_partials;        // block-parallel form: the same, read by the compositor
-    const int32_t *ray_perm;         // ray mode, may be null: thread t marches ray ray_perm[t] (outputs at the ray's index)
+    const int32_t *ray_perm;         // ray mode, may be null: warp t marches ray ray_perm[t] (outputs at the ray's index)
+    const uint32_t *ray_alike;       // ray mode, may be null: rays whose order key is the next ray's
     float *out_block_state;          // ray mode, per-block MLPs, may be null: n_rays x n_ids x 8, per (ray, block
                                      // at its position in ids) C^k (3), F^k (4), the transmittance in front (-1: no sample)
 };
@@ -57,10 +58,15 @@ cudaError_t launch_march_rays(const MarchArgs &a, const RayRecs &rr, cudaStream_
 // A coherent order of a ray batch (ray_order.cu): perm[t] = the ray thread t
 // marches, grouping rays by the cell of their entry into the box [lo, hi]
 // and of their direction.  keys: n scratch words; hist: kRayOrderHistWords
-// words (the bins, then the totals of the scan's blocks of 1024 bins).
+// words (the bins; at kRayOrderAlike the count of rays whose key is the next
+// ray's; the totals of the scan's blocks of 1024 bins).  perm may be null: the
+// count alone.
 constexpr int kRayOrderKeyBits = 18;
 constexpr int kRayOrderBins = 1 << kRayOrderKeyBits;
-constexpr int kRayOrderHistWords = kRayOrderBins + kRayOrderBins / 1024;
+constexpr int kRayOrderAlike = kRayOrderBins;
+constexpr int kRayOrderHistWords = kRayOrderBins + 32 + kRayOrderBins / 1024;
+// Calls of at least this many rays look at the count (launch_march_rays).
+constexpr int64_t kRaysAlikeMin = 1 << 17;
 cudaError_t launch_ray_order(const float *o, const float *d, int64_t n, const float lo[3], const float hi[3],
                              uint32_t *keys, uint32_t *hist, int32_t *perm, cudaStream_t st);
 // Block-parallel form: per-block partials of a ray batch (8 floats per ray
@@ -86,7 +92,7 @@ struct BwdArgs {                  // the call's block records come by value (Ray
     float *partials;              // scratch: backward_rows(n_rays) x 499
     float *gcf;                   // scratch: n_rays x 8 (dL/dC_d, dL/dF per ray)
     unsigned *err;
-    const int32_t *ray_perm;      // may be null: the re-march's thread t takes ray ray_perm[t]
+    const int32_t *ray_perm;      // may be null: the re-march's warp t takes ray ray_perm[t]
 };
 
 // Gradients of the ray-batch form with per-block MLPs (Eq. 5), bwd.cu
@@ -106,7 +112,7 @@ struct BmBwdArgs {                // the call's block records come by value (Ray
     float *S;                     // scratch n_rays x n_ids x 8: C^k (3), F^k (4), B_k (-1: no sample)
     float *G;                     // scratch n_rays x n_ids x 8: dL/dC^k (3), dL/dF^k (4), dL/dC . X_k
     unsigned *err;
-    const int32_t *ray_perm;      // may be null: the marching passes' thread t takes ray ray_perm[t]
+    const int32_t *ray_perm;      // may be null: the marching passes' warp t takes ray ray_perm[t]
     int32_t have_state;           // S already holds the forward's per-block state: skip the first pass
 };
 cudaError_t launch_backward_block_mlps(const BmBwdArgs &a, const RayRecs &rr, cudaStream_t st);

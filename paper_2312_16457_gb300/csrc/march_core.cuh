@@ -333,6 +333,30 @@ __device__ __forceinline__ bool for_each_sample_unbounded(const BlockRec &b, con
     return true;
 }
 
+// Where the ray leaves the empty cell of its sample (the coarse cell around it
+// when that is empty too): the lattice index one step short of the exit, as in
+// for_each_sample.
+__device__ __forceinline__ int empty_exit(const BlockRec &b, const int cell[3], const float o[3], const float d[3],
+                                          const float inv_d[3], float m, float inv_delta) {
+    const int Nc = b.Nc, Nc2 = b.Nc2;
+    const int ci2 = ((cell[2] >> kOccGroupLog2) * Nc2 + (cell[1] >> kOccGroupLog2)) * Nc2 + (cell[0] >> kOccGroupLog2);
+    const int lvl = ((__ldg(b.occ2 + (ci2 >> 5)) >> (ci2 & 31)) & 1u) ? 0 : kOccGroupLog2;
+    const int Ce = b.C << lvl, last = lvl ? Nc2 - 1 : Nc - 1;
+    float tx = 3.0e38f;
+#pragma unroll
+    for (int a = 0; a < 3; a++) {
+        const int ce = cell[a] >> lvl;
+        if (d[a] > 0.f) {
+            const float chi = ce == last ? b.hi[a] : fmaf((float)((ce + 1) * Ce), b.vox[a], b.lo[a]);
+            tx = fminf(tx, (chi - m - o[a]) * inv_d[a]);
+        } else if (d[a] < 0.f) {
+            const float clo = fmaf((float)(ce * Ce), b.vox[a], b.lo[a]);
+            tx = fminf(tx, (clo + m - o[a]) * inv_d[a]);
+        }
+    }
+    return __float2int_rd(tx * inv_delta - 0.5f) - 1;
+}
+
 template <typename Fn>
 __device__ __forceinline__ bool for_each_sample(const BlockRec &b, const float o[3], const float d[3],
                                                 const float inv_d[3], float omax, unsigned *err, Fn &&fn) {
@@ -437,13 +461,11 @@ struct RayState {
     bool done;
 };
 
-// March one ray through one block, updating its state (Eq. 1-2); when tb
-// is given it is multiplied by every sample's 1 - alpha (the block's own
-// transmittance, Eq. 11).
+// March one ray through one block, updating its state (Eq. 1-2).
 template <int DT>
 __device__ __forceinline__ void march_block(const BlockRec &b, const float o[3], const float d[3],
                                             const float inv_d[3], float omax, float ert_eps, RayState &s,
-                                            unsigned *err, float *tb = nullptr) {
+                                            unsigned *err) {
     BrickCache bc;
     const bool more = for_each_sample(b, o, d, inv_d, omax, err, [&](const float p[3], const float g[3], float dt) {
         float2 f2[4];
@@ -457,7 +479,6 @@ __device__ __forceinline__ void march_block(const BlockRec &b, const float o[3],
 #pragma unroll
         for (int c = 0; c < 4; c++) s.F[c] = fmaf(w, sigmoidf_fast(f[4 + c]), s.F[c]);
         s.T *= e;
-        if (tb) *tb *= e;
         s.nsamp++;
         return !(s.T < ert_eps);
     });

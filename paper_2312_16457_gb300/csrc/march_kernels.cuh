@@ -18,6 +18,7 @@
 #include "cow_kernels.h"
 #include "kernel_launch.h"
 #include "march_core.cuh"
+#include "march_warp.cuh"
 
 #ifndef COW_MARCH_MIN_BLOCKS
 #define COW_MARCH_MIN_BLOCKS 4
@@ -26,7 +27,7 @@
 #define COW_MARCH_MIN_BLOCKS_W 4
 #endif
 #ifndef COW_RAYS_MIN_BLOCKS
-#define COW_RAYS_MIN_BLOCKS COW_MARCH_MIN_BLOCKS  // 2 or 3 measured slower on the 2x2-block fit
+#define COW_RAYS_MIN_BLOCKS COW_MARCH_MIN_BLOCKS  // 3 or 5 measured slower on random rays, FP32 and BF16
 #endif
 #ifndef COW_WARP_W
 #define COW_WARP_W 8  // pixels per warp row (the warp covers COW_WARP_W x 32/COW_WARP_W pixels)
@@ -82,27 +83,15 @@ __device__ __forceinline__ int view_of_tile(const MarchArgs &a, int tile) {
 // the ray's total transmittance: inside block k it stops once
 // T_k < ert_eps / T.  rec_at(k) / mlp_at(k): the k-th block's record and
 // MLP weights in near-to-far order.
-// state(k): where the k-th block's state goes (a.out_block_state, ray mode),
-// or null.
-template <int DT, class RecAt, class MlpAt, class StateAt>
+template <int DT, class RecAt, class MlpAt>
 __device__ __forceinline__ void blend_blocks(const MarchArgs &a, int n_blk, RecAt rec_at, MlpAt mlp_at,
-                                             StateAt state, const float o[3], const float d[3],
-                                             const float inv_d[3], float omax, int64_t row) {
+                                             const float o[3], const float d[3], const float inv_d[3], float omax,
+                                             int64_t row) {
     float C[3] = {0.f, 0.f, 0.f}, Cd[3] = {0.f, 0.f, 0.f}, F[4] = {0.f, 0.f, 0.f, 0.f}, T = 1.f;
     int nsamp = 0;
     for (int k = 0; k < n_blk; k++) {
         RayState sb = {{0.f, 0.f, 0.f}, {0.f, 0.f, 0.f, 0.f}, 1.f, 0, false};
         march_block<DT>(rec_at(k), o, d, inv_d, omax, a.ert_eps > 0.f ? a.ert_eps / T : 0.f, sb, a.err);
-        if (float *e = state(k)) {
-            float4 *e4 = reinterpret_cast<float4 *>(e);
-            if (sb.nsamp == 0) {
-                e4[0] = make_float4(0.f, 0.f, 0.f, 0.f);
-                e4[1] = make_float4(0.f, 0.f, 0.f, -1.f);
-            } else {
-                e4[0] = make_float4(sb.Cd[0], sb.Cd[1], sb.Cd[2], sb.F[0]);
-                e4[1] = make_float4(sb.F[1], sb.F[2], sb.F[3], T);
-            }
-        }
         if (sb.nsamp == 0) continue;
         float phi[3];
         block_mlp(mlp_at(k), a.n_freq, sb.Cd, sb.F, d, phi);
@@ -135,8 +124,7 @@ __device__ __forceinline__ void march_blocks_blend(const MarchArgs &a, const Vie
                                                    float omax, int64_t row) {
     blend_blocks<DT>(
         a, v.ids_count, [&](int k) -> const BlockRec & { return recs[k]; },
-        [&](int k) { return a.block_mlps[v.ids_begin + k]; }, [](int) -> float * { return nullptr; }, o, d, inv_d,
-        omax, row);
+        [&](int k) { return a.block_mlps[v.ids_begin + k]; }, o, d, inv_d, omax, row);
 }
 
 // One ray per thread of the tile: march the view's near-to-far block list
@@ -216,116 +204,238 @@ __global__ void __launch_bounds__(kThreads, kMinBlocks)
 }
 
 // ---------------------------------------------------------------------------
-// Warp-per-ray schedule.  A warp marches one ray at a time; lane l takes the
-// lattice sample base + l, so the 32 gathers of one instruction read
-// neighbouring texels of the same ray instead of 32 rays' far-apart texels.
-// The in-block weights of Eq. 1 become an exclusive prefix product of
-// exp(-sigma delta) across the lanes; the transmittance carried across chunks
-// and blocks is Eq. 12-13.  Each lane finally owns one of the warp's 32 rays
-// for the deferred MLP and the output writes.
+// One ray per warp (march_warp.cuh).
 
-__device__ __forceinline__ float warp_exclusive_product(float x, int lane, float &total) {
-    float incl = x;
+// Outputs of the warp's ray: lane c < 7 holds channel c.
+__device__ __forceinline__ void write_outputs_warp(const MarchArgs &a, int64_t row, float acc, float T, int nsamp,
+                                                   float rgb) {
+    const int lane = threadIdx.x & 31;
+    if (lane < 3) a.out_rgb[3 * row + lane] = rgb;
+    if (a.out_aux && lane < 8) a.out_aux[8 * row + lane] = lane < 7 ? acc : T;
+    if (a.out_nsamp && lane == 0) a.out_nsamp[row] = nsamp;
+}
+
+__device__ __forceinline__ void shade_and_write(const MarchArgs &a, int64_t row, const WarpRay &s, const float d[3],
+                                                const float *s_mlp) {
+    float x[10];
 #pragma unroll
-    for (int off = 1; off < 32; off <<= 1) {
-        const float y = __shfl_up_sync(0xffffffffu, incl, off);
-        if (lane >= off) incl *= y;
+    for (int c = 0; c < 7; c++) x[c] = __shfl_sync(kFullMask, s.acc, c);
+#pragma unroll
+    for (int c = 0; c < 3; c++) x[7 + c] = d[c];
+    const float out = deferred_mlp_warp(s_mlp, x, (a.flags & 1u) != 0);
+    write_outputs_warp(a, row, s.acc, s.T, s.nsamp, s.acc + out);
+}
+
+// blend_blocks for the warp's ray.  state(k): where the k-th block's state
+// goes (written for the blocks that are marched), or null.
+template <int DT, class RecAt, class MlpAt, class StateAt>
+__device__ __forceinline__ void blend_blocks_warp(WarpScratch &ws, const MarchArgs &a, int n_blk, RecAt rec_at,
+                                                  MlpAt mlp_at, StateAt state, const float o[3], const float d[3],
+                                                  const float inv_d[3], float omax, int64_t row) {
+    const int lane = threadIdx.x & 31;
+    float C = 0.f, CF = 0.f, T = 1.f;
+    int nsamp = 0;
+    for_each_hit(n_blk, rec_at, o, d, inv_d, [&](int k) {
+        WarpRay sb;
+        march_block_warp<DT>(ws, rec_at(k), o, d, inv_d, omax, a.ert_eps > 0.f ? a.ert_eps / T : 0.f, sb, a.err);
+        if (sb.nsamp == 0) return true;
+        if (float *e = state(k))
+            if (lane < 8) e[lane] = lane < 7 ? sb.acc : T;
+        const float phi = block_mlp_warp(mlp_at(k), a.n_freq, sb.acc, d);
+        C = fmaf(T, sb.acc + phi, C);
+        CF = fmaf(T, sb.acc, CF);
+        T *= sb.T;
+        nsamp += sb.nsamp;
+        return !sb.done;
+    });
+    write_outputs_warp(a, row, CF, T, nsamp, C);
+}
+
+// A camera's rays given as a ray batch: three quarters of them enter where the
+// next ray enters, in its direction (32 consecutive rays can have 31 such).
+__device__ __forceinline__ bool rays_alike(const MarchArgs &a) {
+    return a.ray_alike && 4 * (int64_t)__ldg(a.ray_alike) >= 3 * a.n_rays;
+}
+
+// The ray form for such rays, one ray per thread in the given order: the rays
+// of a warp are neighbouring pixels, and their gathers share lines as the view
+// marcher's do (16 blocks of 128^3 FP16, the 921600 rays of a 720p camera: 9.2
+// ms, one ray per warp 13.4 ms).
+template <int DT, bool kBlockMlp>
+__global__ void __launch_bounds__(kThreads, kMinBlocks) k_march_rays_t(const __grid_constant__ MarchArgs a,
+                                                                       const __grid_constant__ RayRecs rr) {
+    __shared__ float s_mlp[kMlpParams + 1];
+    if (!rays_alike(a)) return;
+    if (!kBlockMlp) {
+        load_mlp(a.mlp, s_mlp, (a.flags & 1u) != 0);
+        __syncthreads();
     }
-    total = __shfl_sync(0xffffffffu, incl, 31);
-    const float ex = __shfl_up_sync(0xffffffffu, incl, 1);
-    return lane == 0 ? 1.0f : ex;
-}
-
-__device__ __forceinline__ float warp_sum(float x) {
+    const int64_t r = (int64_t)blockIdx.x * kThreads + threadIdx.x;
+    if (r >= a.n_rays) return;
+    float o[3], d[3];
 #pragma unroll
-    for (int off = 16; off > 0; off >>= 1) x += __shfl_xor_sync(0xffffffffu, x, off);
-    return x;
+    for (int c = 0; c < 3; c++) {
+        o[c] = __ldg(a.ray_o + 3 * r + c);
+        d[c] = __ldg(a.ray_d + 3 * r + c);
+    }
+    int order[kMaxRayIds];
+    const int n = sort_blocks_for_ray(rr, o, order);
+    float inv_d[3], omax;
+    ray_setup(d, o, inv_d, omax);
+    if (kBlockMlp) {
+        blend_blocks<DT>(
+            a, n, [&](int k) -> const BlockRec & { return rr.r[order[k]]; },
+            [&](int k) { return a.block_mlp_base + (int64_t)rr.id[order[k]] * a.block_mlp_stride; }, o, d, inv_d, omax,
+            r);
+        return;
+    }
+    RayState s = {{0.f, 0.f, 0.f}, {0.f, 0.f, 0.f, 0.f}, 1.f, 0, false};
+    for (int k = 0; k < n && !s.done; k++)
+        march_block<DT>(rr.r[order[k]], o, d, inv_d, omax, a.ert_eps, s, a.err);
+    write_outputs(a, r, s, d, s_mlp);
 }
 
+template <int DT, bool kBlockMlp>
+__global__ void __launch_bounds__(kThreads, COW_RAYS_MIN_BLOCKS) k_march_rays(const __grid_constant__ MarchArgs a,
+                                                                          const __grid_constant__ RayRecs rr) {
+    __shared__ float s_mlp[kMlpParams + 1];
+    __shared__ WarpScratch s_ws[kThreads / 32];
+    if (rays_alike(a)) return;  // k_march_rays_t has them
+    if (!kBlockMlp) {
+        load_mlp(a.mlp, s_mlp, (a.flags & 1u) != 0);
+        __syncthreads();
+    }
+    WarpScratch &ws = s_ws[threadIdx.x >> 5];
+    const int lane = threadIdx.x & 31;
+    float o[3], d[3], inv_d[3], omax;
+    const int64_t r = load_ray_warp(a, o, d);
+    if (r < 0) return;
+    ray_setup(d, o, inv_d, omax);
+    // per-ray depth order: xy distance of block centres to this origin (App. D)
+    const int n = sort_blocks_warp(ws, rr, o);
+    auto rec_at = [&](int k) -> const BlockRec & { return rr.r[ws.ord[k]]; };
+    if (kBlockMlp) {  // Eq. 5 with block id's own MLP at block_mlp_base + id * block_mlp_stride
+        float *bs = a.out_block_state ? a.out_block_state + 8 * r * n : nullptr;
+        if (bs) {  // blocks without an occupied sample
+            for (int k = lane; k < 8 * n; k += 32) bs[k] = (k & 7) == 7 ? -1.f : 0.f;
+            __syncwarp();
+        }
+        blend_blocks_warp<DT>(
+            ws, a, n, rec_at,
+            [&](int k) { return a.block_mlp_base + (int64_t)rr.id[ws.ord[k]] * a.block_mlp_stride; },
+            [&](int k) -> float * { return bs ? bs + 8 * ws.ord[k] : nullptr; }, o, d, inv_d, omax, r);
+        return;
+    }
+    WarpRay s;
+    if (a.out_block_T) {
+        // also every block's own transmittance, at its position in ids; -1
+        // for a block without occupied samples (the call has no early
+        // termination, so every block is marched)
+        float *bt = a.out_block_T + r * n;
+        for (int k = lane; k < n; k += 32) bt[k] = -1.f;
+        __syncwarp();
+        for_each_hit(n, rec_at, o, d, inv_d, [&](int k) {
+            float tb = 1.f;
+            const int n0 = s.nsamp;
+            march_block_warp<DT>(ws, rec_at(k), o, d, inv_d, omax, a.ert_eps, s, a.err, &tb);
+            if (lane == 0 && s.nsamp > n0) bt[ws.ord[k]] = tb;
+            return true;
+        });
+    } else {
+        for_each_hit(n, rec_at, o, d, inv_d, [&](int k) {
+            march_block_warp<DT>(ws, rec_at(k), o, d, inv_d, omax, a.ert_eps, s, a.err);
+            return !s.done;
+        });
+    }
+    shade_and_write(a, r, s, d, s_mlp);
+}
+
+// Block-parallel form, first half: every block of the call marched on its
+// own from an in-block transmittance of 1 (Eq. 11: C_d^k, F^k and T^k =
+// 1 - alpha^k of block k alone), written as 8 floats per (ray, block) in
+// the order of the call's ids.  No early termination (a partial must not
+// depend on the blocks in front of it).
 template <int DT>
-__device__ __forceinline__ void march_block_warp(const BlockRec &b, const float o[3], const float d[3],
-                                                 const float inv_d[3], float omax, float ert_eps, int lane,
-                                                 float &T, float pc[3], float pf[4], int &nsamp, bool &done,
-                                                 unsigned *err) {
-    int i0, i1;
-    float tfar;
-    if (!candidate_range(b, o, d, inv_d, i0, i1, tfar)) return;
-    if (i1 - i0 > kMaxSpan) {
-        if (lane == 0) atomicOr(err, kErrRange);
-        i1 = i0 + kMaxSpan;
-    }
-    const float delta = b.delta, inv_delta = 1.0f / b.delta;
-    const float m = 4e-6f * (omax + tfar + b.bmax);
-    const int Nc = b.Nc, C = b.C, R = b.R;
-    for (int base = i0; base <= i1;) {
-        const int i = base + lane;
-        bool inb = false, occ = false;
-        float p[3], g[3];
-        int cell[3] = {0, 0, 0};
-        if (i <= i1) {
-            lattice_point(o, d, delta, i, p);
-            inb = inside_block(b, p);
-            if (inb) {
-#pragma unroll
-                for (int a = 0; a < 3; a++) {
-                    g[a] = axis_coord(p[a], b.lo[a], b.kg[a]);
-                    const int v = min(max(__float2int_rd(g[a]), 0), R - 2);
-                    cell[a] = C == 1 ? v : (int)__umulhi((unsigned)v, b.cdiv);
-                }
-                const int ci = (cell[2] * Nc + cell[1]) * Nc + cell[0];
-                occ = (__ldg(b.occ + (ci >> 5)) >> (ci & 31)) & 1u;
-            }
-        }
-        float e = 1.f, c[7];
-        if (occ) {
-            float2 f2[4];
-            BrickCache bc;  // one lattice sample of this lane: the brick is stored
-            accumulate_sample<DT>(b, p, g, f2, &bc);
-            const float f[8] = {f2[0].x, f2[0].y, f2[1].x, f2[1].y, f2[2].x, f2[2].y, f2[3].x, f2[3].y};
-            e = __expf(-__expf(f[0]) * delta);
-#pragma unroll
-            for (int k = 0; k < 7; k++) c[k] = sigmoidf_fast(f[1 + k]);
-        }
-        float chunk;
-        const float ex = warp_exclusive_product(e, lane, chunk);
-        if (occ) {
-            const float w = (T * ex) * (1.f - e);
-#pragma unroll
-            for (int k = 0; k < 3; k++) pc[k] = fmaf(w, c[k], pc[k]);
-#pragma unroll
-            for (int k = 0; k < 4; k++) pf[k] = fmaf(w, c[3 + k], pf[k]);
-        }
-        T *= chunk;
-        nsamp += __popc(__ballot_sync(0xffffffffu, occ));
-        // next chunk: past lane 31's empty cell when it sits in one (exact, as in the thread schedule)
-        int j = -1;
-        if (lane == 31 && inb && !occ) {
-            float tx = 3.0e38f;
-#pragma unroll
-            for (int a = 0; a < 3; a++) {
-                if (d[a] > 0.f) {
-                    const float chi =
-                        cell[a] == Nc - 1 ? b.hi[a] : fmaf((float)((cell[a] + 1) * C), b.vox[a], b.lo[a]);
-                    tx = fminf(tx, (chi - m - o[a]) * inv_d[a]);
-                } else if (d[a] < 0.f) {
-                    const float clo = fmaf((float)(cell[a] * C), b.vox[a], b.lo[a]);
-                    tx = fminf(tx, (clo + m - o[a]) * inv_d[a]);
-                }
-            }
-            j = __float2int_rd(tx * inv_delta - 0.5f) - 1;
-        }
-        j = __shfl_sync(0xffffffffu, j, 31);
-        base = max(base + 32, j + 1);
-        if (T < ert_eps) {
-            done = true;
-            return;
-        }
-    }
+__global__ void __launch_bounds__(kThreads, COW_RAYS_MIN_BLOCKS) k_march_partials(const __grid_constant__ MarchArgs a,
+                                                                              const __grid_constant__ RayRecs rr) {
+    __shared__ WarpScratch s_ws[kThreads / 32];
+    WarpScratch &ws = s_ws[threadIdx.x >> 5];
+    const int lane = threadIdx.x & 31;
+    float o[3], d[3], inv_d[3], omax;
+    const int64_t r = load_ray_warp(a, o, d);
+    if (r < 0) return;
+    ray_setup(d, o, inv_d, omax);
+    float *pp = a.out_partials + 8 * r * rr.n;
+    for (int k = lane; k < 8 * rr.n; k += 32) pp[k] = (k & 7) == 7 ? 1.f : 0.f;
+    __syncwarp();
+    for_each_hit(rr.n, [&](int k) -> const BlockRec & { return rr.r[k]; }, o, d, inv_d, [&](int k) {
+        WarpRay s;
+        march_block_warp<DT>(ws, rr.r[k], o, d, inv_d, omax, 0.f, s, a.err);
+        if (lane < 8) pp[8 * k + lane] = lane < 7 ? s.acc : s.T;
+        return true;
+    });
 }
 
+// Frames of up to this many pixels are marched one ray per warp: one ray per
+// thread then has every ray on the chip at once (152 SMs x 512 threads) and
+// takes as long as its longest ray.  Measured (us, thread / warp form): M = 1
+// block of 64^3 FP32, 128x128 357 / 98, 320x240 389 / 337, 400x300 488 / 525;
+// 4x4 blocks of 128^3 BF16, 96x54 2585 / 125, 320x240 2223 / 1382, 400x300
+// 2286 / 2113, 480x360 2662 / 2996; three-level city BF16, 96x54 2985 / 83,
+// 320x240 1885 / 666.
+constexpr int64_t kChipRays = 152 * kMinBlocks * kThreads;
+
+// One ray per warp over a view's near-to-far block list.
+template <int DT, bool kBlockMlp>
+__device__ __forceinline__ void march_pixel_warp(WarpScratch &ws, const MarchArgs &a, const ViewRec &v,
+                                                 const BlockRec *recs, int px, int py, const float *s_mlp) {
+    if (px >= v.W || py >= v.H) return;  // uniform across the warp
+    float o[3], d[3], inv_d[3], omax;
+    pixel_ray(v, px, py, o, d);
+    ray_setup(d, o, inv_d, omax);
+    const int64_t row = v.pix_offset + (int64_t)py * v.W + px;
+    auto rec_at = [&](int k) -> const BlockRec & { return recs[k]; };
+    if (kBlockMlp) {
+        blend_blocks_warp<DT>(
+            ws, a, v.ids_count, rec_at, [&](int k) { return a.block_mlps[v.ids_begin + k]; },
+            [](int) -> float * { return nullptr; }, o, d, inv_d, omax, row);
+        return;
+    }
+    WarpRay s;
+    for_each_hit(v.ids_count, rec_at, o, d, inv_d, [&](int k) {
+        march_block_warp<DT>(ws, recs[k], o, d, inv_d, omax, a.ert_eps, s, a.err);
+        return !s.done;
+    });
+    shade_and_write(a, row, s, d, s_mlp);
+}
+
+// Small frames, records in the parameter buffer: a CTA takes a 2x2 patch of a
+// 16x8 tile, one pixel per warp.
+template <int DT, bool kBlockMlp>
+__global__ void __launch_bounds__(kThreads, kMinBlocksW)
+    k_march_views_cw(const __grid_constant__ MarchArgs a, const __grid_constant__ ParamRecs pr) {
+    __shared__ float s_mlp[kMlpParams + 1];
+    __shared__ WarpScratch s_ws[kThreads / 32];
+    const int tile = blockIdx.x >> 5, sub = blockIdx.x & 31;
+    const ViewRec &v = a.views[view_of_tile(a, tile)];
+    int tx, ty;
+    tile_xy(v, tile - v.tile_begin, kTileH, tx, ty);
+    const int px0 = tx * kTileW + 2 * (sub & 7), py0 = ty * kTileH + 2 * (sub >> 3);
+    if (px0 >= v.W || py0 >= v.H) return;
+    if (!kBlockMlp) {
+        load_mlp(a.mlp, s_mlp, (a.flags & 1u) != 0);
+        __syncthreads();
+    }
+    const int warp = threadIdx.x >> 5;
+    march_pixel_warp<DT, kBlockMlp>(s_ws[warp], a, v, pr.r + v.ids_begin, px0 + (warp & 1), py0 + (warp >> 1), s_mlp);
+}
+
+// COW_SCHED_WARP: the tile's rays one after another, 32 per warp, records in
+// shared memory.
 template <int DT>
 __global__ void __launch_bounds__(kThreads, kMinBlocksW) k_march_views_w(MarchArgs a) {
     __shared__ float s_mlp[kMlpParams + 1];
+    __shared__ WarpScratch s_ws[kThreads / 32];
     __shared__ alignas(16) BlockRec s_rec[kMaxSmemRecs];
     __shared__ alignas(8) uint64_t s_bar;
     const int tile = blockIdx.x;
@@ -343,130 +453,15 @@ __global__ void __launch_bounds__(kThreads, kMinBlocksW) k_march_views_w(MarchAr
             atomicOr(a.err, kErrTimeout);
             if (!mbar_wait(&s_bar, 0, polls)) return;
         }
+        __syncwarp();
     }
     const BlockRec *recs = staged ? s_rec : a.recs + v.ids_begin;
-    const int t = tile - v.tile_begin;
     int tx, ty;
-    tile_xy(v, t, kTileH, tx, ty);
-    const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+    tile_xy(v, tile - v.tile_begin, kTileH, tx, ty);
+    const int warp = threadIdx.x >> 5;
     const int px0 = tx * kTileW + (warp & 1) * 8, py0 = ty * kTileH + (warp >> 1) * 4;
-    // this lane's own ray (it writes its outputs at the end)
-    const int px = px0 + (lane & 7), py = py0 + (lane >> 3);
-    const bool mine_valid = px < v.W && py < v.H;
-    float mo[3], md[3];
-    pixel_ray(v, min(px, v.W - 1), min(py, v.H - 1), mo, md);
-    float my_acc[8] = {0.f, 0.f, 0.f, 0.f, 0.f, 0.f, 0.f, 1.f};
-    int my_n = 0;
-    for (int q = 0; q < 32; q++) {
-        const int qx = px0 + (q & 7), qy = py0 + (q >> 3);
-        if (qx >= v.W || qy >= v.H) continue;  // uniform across the warp
-        float o[3], d[3], inv_d[3], omax;
-#pragma unroll
-        for (int k = 0; k < 3; k++) {
-            o[k] = __shfl_sync(0xffffffffu, mo[k], q);
-            d[k] = __shfl_sync(0xffffffffu, md[k], q);
-        }
-        ray_setup(d, o, inv_d, omax);
-        float T = 1.f, pc[3] = {0.f, 0.f, 0.f}, pf[4] = {0.f, 0.f, 0.f, 0.f};
-        int nsamp = 0;
-        bool done = false;
-        for (int k = 0; k < n_blk && !done; k++)
-            march_block_warp<DT>(recs[k], o, d, inv_d, omax, a.ert_eps, lane, T, pc, pf, nsamp, done, a.err);
-        float tot[7];
-#pragma unroll
-        for (int k = 0; k < 3; k++) tot[k] = warp_sum(pc[k]);
-#pragma unroll
-        for (int k = 0; k < 4; k++) tot[3 + k] = warp_sum(pf[k]);
-        if (lane == q) {
-#pragma unroll
-            for (int k = 0; k < 7; k++) my_acc[k] = tot[k];
-            my_acc[7] = T;
-            my_n = nsamp;
-        }
-    }
-    if (!mine_valid) return;
-    RayState s = {{my_acc[0], my_acc[1], my_acc[2]}, {my_acc[3], my_acc[4], my_acc[5], my_acc[6]}, my_acc[7], my_n,
-                  false};
-    write_outputs(a, v.pix_offset + (int64_t)py * v.W + px, s, md, s_mlp);
-}
-
-template <int DT, bool kBlockMlp>
-__global__ void __launch_bounds__(kThreads, COW_RAYS_MIN_BLOCKS) k_march_rays(MarchArgs a,
-                                                                          const __grid_constant__ RayRecs rr) {
-    __shared__ float s_mlp[kMlpParams + 1];
-    if (!kBlockMlp) {
-        load_mlp(a.mlp, s_mlp, (a.flags & 1u) != 0);
-        __syncthreads();
-    }
-    const int64_t t = (int64_t)blockIdx.x * kThreads + threadIdx.x;
-    if (t >= a.n_rays) return;
-    const int64_t r = a.ray_perm ? (int64_t)__ldg(a.ray_perm + t) : t;
-    float o[3], d[3];
-#pragma unroll
-    for (int c = 0; c < 3; c++) {
-        o[c] = __ldg(a.ray_o + 3 * r + c);
-        d[c] = __ldg(a.ray_d + 3 * r + c);
-    }
-    // per-ray depth order: xy distance of block centres to this origin (App. D)
-    int order[kMaxRayIds];
-    const int n = sort_blocks_for_ray(rr, o, order);
-    float inv_d[3], omax;
-    ray_setup(d, o, inv_d, omax);
-    if (kBlockMlp) {  // Eq. 5 with block id's own MLP at block_mlp_base + id * block_mlp_stride
-        blend_blocks<DT>(
-            a, n, [&](int k) -> const BlockRec & { return rr.r[order[k]]; },
-            [&](int k) { return a.block_mlp_base + (int64_t)rr.id[order[k]] * a.block_mlp_stride; },
-            [&](int k) -> float * {
-                return a.out_block_state ? a.out_block_state + 8 * (r * rr.n + order[k]) : nullptr;
-            },
-            o, d, inv_d, omax, r);
-        return;
-    }
-    RayState s = {{0.f, 0.f, 0.f}, {0.f, 0.f, 0.f, 0.f}, 1.f, 0, false};
-    if (a.out_block_T) {
-        // also every block's own transmittance, at its position in ids; -1
-        // for a block without occupied samples (the call has no early
-        // termination, so every block is marched)
-        float *bt = a.out_block_T + r * n;
-        for (int k = 0; k < n; k++) {
-            float tb = 1.f;
-            const int n0 = s.nsamp;
-            march_block<DT>(rr.r[order[k]], o, d, inv_d, omax, a.ert_eps, s, a.err, &tb);
-            bt[order[k]] = s.nsamp > n0 ? tb : -1.f;
-        }
-    } else {
-        for (int k = 0; k < n && !s.done; k++)
-            march_block<DT>(rr.r[order[k]], o, d, inv_d, omax, a.ert_eps, s, a.err);
-    }
-    write_outputs(a, r, s, d, s_mlp);
-}
-
-// Block-parallel form, first half: every block of the call marched on its
-// own from an in-block transmittance of 1 (Eq. 11: C_d^k, F^k and T^k =
-// 1 - alpha^k of block k alone), written as 8 floats per (ray, block) in
-// the order of the call's ids.  No early termination (a partial must not
-// depend on the blocks in front of it).
-template <int DT>
-__global__ void __launch_bounds__(kThreads, COW_RAYS_MIN_BLOCKS) k_march_partials(MarchArgs a,
-                                                                              const __grid_constant__ RayRecs rr) {
-    const int64_t t = (int64_t)blockIdx.x * kThreads + threadIdx.x;
-    if (t >= a.n_rays) return;
-    const int64_t r = a.ray_perm ? (int64_t)__ldg(a.ray_perm + t) : t;
-    float o[3], d[3];
-#pragma unroll
-    for (int c = 0; c < 3; c++) {
-        o[c] = __ldg(a.ray_o + 3 * r + c);
-        d[c] = __ldg(a.ray_d + 3 * r + c);
-    }
-    float inv_d[3], omax;
-    ray_setup(d, o, inv_d, omax);
-    for (int k = 0; k < rr.n; k++) {
-        RayState s = {{0.f, 0.f, 0.f}, {0.f, 0.f, 0.f, 0.f}, 1.f, 0, false};
-        march_block<DT>(rr.r[k], o, d, inv_d, omax, 0.f, s, a.err);
-        float4 *pp = reinterpret_cast<float4 *>(a.out_partials + 8 * (r * rr.n + k));
-        pp[0] = make_float4(s.Cd[0], s.Cd[1], s.Cd[2], s.F[0]);
-        pp[1] = make_float4(s.F[1], s.F[2], s.F[3], s.T);
-    }
+    for (int q = 0; q < 32; q++)
+        march_pixel_warp<DT, false>(s_ws[warp], a, v, recs, px0 + (q & 7), py0 + (q >> 3), s_mlp);
 }
 
 template <int DT, bool kBlockMlp>
@@ -496,13 +491,23 @@ cudaError_t launch_views_dt(const MarchArgs &a, int n_tiles, int schedule, cudaS
     }
     const bool in_params = schedule == kSchedThreadConst;
     if (in_params && !pr) return cudaErrorInvalidValue;
+    if (in_params && a.n_rays <= kChipRays) {
+        if (block_mlp) k_march_views_cw<DT, true><<<n_tiles * 32, kThreads, 0, st>>>(a, *pr);
+        else k_march_views_cw<DT, false><<<n_tiles * 32, kThreads, 0, st>>>(a, *pr);
+        return cudaGetLastError();
+    }
     return block_mlp ? launch_thread<DT, true>(a, n_tiles, in_params, st, pr)
                      : launch_thread<DT, false>(a, n_tiles, in_params, st, pr);
 }
 
 template <int DT>
 cudaError_t launch_rays_dt(const MarchArgs &a, const RayRecs &rr, cudaStream_t st) {
-    const int64_t nb = (a.n_rays + kThreads - 1) / kThreads;
+    const int64_t nb = (a.n_rays + kThreads / 32 - 1) / (kThreads / 32);
+    if (a.ray_alike) {  // decided on the device by the count of alike rays: the other of the two kernels returns at once
+        const unsigned nt = (unsigned)((a.n_rays + kThreads - 1) / kThreads);
+        if (a.block_mlp_base) k_march_rays_t<DT, true><<<nt, kThreads, 0, st>>>(a, rr);
+        else k_march_rays_t<DT, false><<<nt, kThreads, 0, st>>>(a, rr);
+    }
     if (a.block_mlp_base) k_march_rays<DT, true><<<(unsigned)nb, kThreads, 0, st>>>(a, rr);
     else k_march_rays<DT, false><<<(unsigned)nb, kThreads, 0, st>>>(a, rr);
     return cudaGetLastError();
@@ -510,7 +515,7 @@ cudaError_t launch_rays_dt(const MarchArgs &a, const RayRecs &rr, cudaStream_t s
 
 template <int DT>
 cudaError_t launch_partials_dt(const MarchArgs &a, const RayRecs &rr, cudaStream_t st) {
-    const int64_t nb = (a.n_rays + kThreads - 1) / kThreads;
+    const int64_t nb = (a.n_rays + kThreads / 32 - 1) / (kThreads / 32);
     k_march_partials<DT><<<(unsigned)nb, kThreads, 0, st>>>(a, rr);
     return cudaGetLastError();
 }
