@@ -1,12 +1,12 @@
 // bwd.cu -- K6 / K7: gradients of the rendered colour with respect to every
 // grid, plane and deferred-MLP parameter, for the ray-batch form.
 //
-// Per ray (one thread), given g = dL/dC:
+// Per ray, given g = dL/dC:
 //   K7  recompute the deferred MLP (Eq. 3) from the forward's saved C_d, F and
 //       back-propagate it: dL/dC_d = g + dPhi/dC_d^T g, dL/dF, and the ray's
 //       contribution to dL/dW (outer products kept in shared memory).
-//   K6  re-march the ray over exactly the forward's samples (same sequence
-//       code) with the transmittance T and the running prefix sums P_C, P_F;
+//   K6  (one ray per warp, march_warp.cuh) re-march the ray over exactly the
+//       forward's samples (same sequence code) with the transmittance T and the running prefix sums P_C, P_F;
 //       the contribution of the samples after i is the saved total minus the
 //       prefix, so no sample is stored.  With e = 1 - alpha = exp(-sigma delta)
 //       and the weights of Eq. 1 (w_i = T_i alpha_i):
@@ -16,24 +16,30 @@
 //                 = sigma delta (T_i e_i (gC.c_i + gF.s_i) - (gC.S_C + gF.S_F))
 //       (no division), then dL/df = dL/df0, c(1-c) dL/dc, s(1-s) dL/ds is
 //       scattered with the interpolation weights to the 8 grid vertices and
-//       12 plane texels (float4 atomics into FP32 gradient arrays in the
+//       12 plane texels (float4 reductions into FP32 gradient arrays in the
 //       natural layout).
+// K6's bound was the L2's rate of scattered reductions, 40 float4 a sample (one
+// ray per thread: 130 ms for 2^20 random rays over 2x2 blocks of 128^3 FP32,
+// 5.5e8 samples).  With a voxel's or texel's contributions added up before they
+// are reduced and the reductions in 64-byte groups it takes 73 ms; what bounds
+// it now is latency at 16 warps per SM (issue slots 37 % busy) with the L1 data
+// pipe 63 % and the L2 53 % busy, gathers and reductions together.
 // The CTA's MLP weight gradient (499 sums over its 128 rays) goes to a
 // per-CTA scratch row; a second kernel adds the rows in a fixed order, so the
 // MLP gradient does not depend on scheduling.
 #include "cow_common.cuh"
 #include "cow_kernels.h"
 #include "march_core.cuh"
+#include "march_warp.cuh"
 
 namespace cow {
 
 namespace {
 
 #ifndef COW_BWD_MIN_BLOCKS
-// CTAs per SM the re-march's register budget is sized for: 2 lets it keep its
-// ~168 live registers (the compiler's own choice, 128, spills); measured on
-// the 2x2-block fit: 2 -> 296 ms a step, 3 -> 300, 4 or unset -> 312
-#define COW_BWD_MIN_BLOCKS 2
+// CTAs per SM the re-march's register budget is sized for: the 2^20-ray step
+// takes 142 ms at 2, 120 at 3, 107 at 4 and 106 at 5, which spills 80 bytes
+#define COW_BWD_MIN_BLOCKS 4
 #endif
 
 #ifndef COW_REG_MIN_BLOCKS
@@ -43,6 +49,7 @@ namespace {
 #endif
 
 constexpr int kBwdThreads = kBwdCtaThreads;
+constexpr int kBwdWarps = kBwdThreads / 32;
 constexpr int kVec = 77;  // x (10), dz1 (16), h1 (16), dz2 (16), h2 (16), dz3 (3)
 
 // Vector reduction without a returned value (red, not atom: a float4
@@ -57,55 +64,224 @@ __device__ __forceinline__ void red_add1(float *dst, float a) {
     asm volatile("red.global.add.f32 [%0], %1;" ::"l"(dst), "f"(a) : "memory");
 }
 
-__device__ __forceinline__ void red_add8(float *dst, float s, const float gf[8]) {
-    red_add4(dst, s * gf[0], s * gf[1], s * gf[2], s * gf[3]);
-    red_add4(dst + 4, s * gf[4], s * gf[5], s * gf[6], s * gf[7]);
+// One sample's feature gradient and where it goes, in shared memory while the
+// warp scatters a chunk.
+struct alignas(16) TapRec {
+    float fr[3];        // place inside the voxel
+    uint32_t base_lo;   // the voxel's first vertex
+    float hf[3];        // places inside the texel cells along x, y, z
+    uint32_t base_hi;
+    uint32_t texel[4];  // first texel of the xy, xz, yz footprints; unused
+    float gf[8];
+};
+
+// Shared scratch of one warp of the re-march.
+struct alignas(16) BwdScratch {
+    WarpScratch w;
+    float T[kRowPad];  // transmittance in front of the chunk's samples
+    TapRec tap[32];
+};
+
+// Bits j of a chunk's first n samples after which a run of equal keys ends.
+// `same`: this lane's key equals the previous lane's.
+__device__ __forceinline__ unsigned run_ends(bool same, int n) {
+    const unsigned starts = __ballot_sync(kFullMask, !same);
+    return ((starts >> 1) | (1u << (n - 1))) & (kFullMask >> (32 - n));
 }
 
-// Scatter an 8-channel feature gradient to the taps of the lookup at (p, g).
-__device__ __forceinline__ void scatter_taps(const BlockRec &b, float *gg, float *const gp[3], const float p[3],
-                                             const float g[3], const float gf[8]) {
-    float fr[3];
-    int c0[3];
+// acc += w v over the four channels of a half
+__device__ __forceinline__ void add_half(float2 acc[2], float w, const float4 &v) {
+    const float2 w2 = make_float2(w, w);
+    acc[0] = __ffma2_rn(w2, make_float2(v.x, v.y), acc[0]);
+    acc[1] = __ffma2_rn(w2, make_float2(v.z, v.w), acc[1]);
+}
+
+__device__ __forceinline__ void flush_half(float *dst, float2 acc[2]) {
+    red_add4(dst, acc[0].x, acc[0].y, acc[1].x, acc[1].y);
+    acc[0] = acc[1] = make_float2(0.f, 0.f);
+}
+
+// Scatter a chunk of n samples (lane j < n holds sample j's point and gradient
+// gf) to the taps of their lookups, as a warp: a lane has one tap and one half
+// of its eight channels, so the lanes of one reduction cover whole 64-byte
+// vertex or texel pairs (the L2 takes 64-byte groups of float4 reductions 1.6
+// times as fast as scattered ones: 330 against 205 G/s into 32 MiB, 147 against
+// 46 G/s into 256 MiB), and it walks its samples in ray order, adding up what
+// goes to one voxel or texel cell before it issues the reduction (a lattice
+// step is about a quarter of a voxel, so a voxel takes some 2.5 samples).
+__device__ __forceinline__ void scatter_chunk(const BlockRec &b, TapRec *tap, int n, const float p[3],
+                                              const float g[3], const float gf[8], float *gg, float *const gp[3]) {
+    const int lane = threadIdx.x & 31;
+    uint64_t base = 0;
+    uint32_t tx[3] = {0, 0, 0};
+    if (lane < n) {
+        int c0[3], h0[3];
+        float fr[3], hf[3];
 #pragma unroll
-    for (int a = 0; a < 3; a++) {
-        const int v = min(max(__float2int_rd(g[a]), 0), b.R - 2);
-        c0[a] = v;
-        fr[a] = fminf(fmaxf(g[a], 0.f), (float)(b.R - 1)) - (float)v;
+        for (int a = 0; a < 3; a++) {
+            c0[a] = min(max(__float2int_rd(g[a]), 0), b.R - 2);
+            fr[a] = fminf(fmaxf(g[a], 0.f), (float)(b.R - 1)) - (float)c0[a];
+            const float h = axis_coord(p[a], b.plo[a], b.kp[a]);
+            h0[a] = min(max(__float2int_rd(h), 0), b.P - 2);
+            hf[a] = fminf(fmaxf(h, 0.f), (float)(b.P - 1)) - (float)h0[a];
+        }
+        base = ((uint64_t)c0[2] * b.R + c0[1]) * b.R + c0[0];
+        // below 2^32: a plane of more texels, with its gradient, exceeds the device
+        tx[0] = (uint32_t)h0[1] * b.P + h0[0];
+        tx[1] = (uint32_t)h0[2] * b.P + h0[0];
+        tx[2] = (uint32_t)h0[2] * b.P + h0[1];
+        float4 *o = reinterpret_cast<float4 *>(tap + lane);
+        o[0] = make_float4(fr[0], fr[1], fr[2], __uint_as_float((uint32_t)base));
+        o[1] = make_float4(hf[0], hf[1], hf[2], __uint_as_float((uint32_t)(base >> 32)));
+        o[2] = make_float4(__uint_as_float(tx[0]), __uint_as_float(tx[1]), __uint_as_float(tx[2]), 0.f);
+        o[3] = make_float4(gf[0], gf[1], gf[2], gf[3]);
+        o[4] = make_float4(gf[4], gf[5], gf[6], gf[7]);
     }
-    const int64_t R = b.R;
-    const int64_t base = (c0[2] * R + c0[1]) * R + c0[0];
-    const float wx[2] = {1.f - fr[0], fr[0]}, wy[2] = {1.f - fr[1], fr[1]}, wz[2] = {1.f - fr[2], fr[2]};
-    if (gg) {
+    const uint64_t pbase = __shfl_up_sync(kFullMask, base, 1);
+    unsigned ends = run_ends(pbase == base && lane > 0, n);
+    unsigned pends[3];
 #pragma unroll
-        for (int k = 0; k < 8; k++) {
-            const int dx = k & 1, dy = (k >> 1) & 1, dz = k >> 2;
-            red_add8(gg + 8 * (base + (dz * R + dy) * R + dx), (wy[dy] * wz[dz]) * wx[dx], gf);
+    for (int k = 0; k < 3; k++) {
+        const uint32_t ptx = __shfl_up_sync(kFullMask, tx[k], 1);
+        pends[k] = run_ends(ptx == tx[k] && lane > 0, n);
+    }
+    __syncwarp();
+    // place q (0 or 1) of an axis: weight 1 - f or f, as s f + c
+    const float s1 = (lane & 2) ? 1.f : -1.f, c1 = (lane & 2) ? 0.f : 1.f;
+    const float s2 = (lane & 4) ? 1.f : -1.f, c2 = (lane & 4) ? 0.f : 1.f;
+    const int half = 4 * (lane & 1);
+    const bool a1 = lane & 2, a2 = lane & 4;
+    if (gg) {  // two runs of samples, 16 lanes each: 8 vertices x 2 halves
+        const float s3 = (lane & 8) ? 1.f : -1.f, c3 = (lane & 8) ? 0.f : 1.f;
+        const int64_t R = b.R;
+        float *const dst = gg + 8 * (((lane & 8 ? R : 0) + (a2 ? 1 : 0)) * R + (a1 ? 1 : 0)) + half;
+        const int len = (n + 1) >> 1, j0 = (lane >> 4) * len;
+        ends |= 1u << (len - 1);
+        const unsigned mine = ends >> j0;
+        const TapRec *t = tap + j0;
+        float2 acc[2] = {make_float2(0.f, 0.f), make_float2(0.f, 0.f)};
+#pragma unroll 2
+        for (int j = 0; j < len; j++) {
+            const float4 f = *reinterpret_cast<const float4 *>(t[j].fr);
+            const float4 v = *reinterpret_cast<const float4 *>(t[j].gf + half);
+            add_half(acc, (fmaf(f.y, s2, c2) * fmaf(f.z, s3, c3)) * fmaf(f.x, s1, c1), v);
+            if ((mine >> j) & 1u)
+                flush_half(dst + 8 * ((uint64_t)t[j].base_hi << 32 | __float_as_uint(f.w)), acc);
         }
     }
-    float hf[3];
-    int h0[3];
+    // four runs, 8 lanes each: per plane 4 texels x 2 halves
+    const int len = (n + 3) >> 2, j0 = (lane >> 3) * len;
+    const unsigned cuts = ((1u << (len - 1)) | (1u << (2 * len - 1)) | (1u << (3 * len - 1))) & (kFullMask >> (32 - n));
+    const TapRec *t = tap + j0;
+    const uint32_t off = (a2 ? b.P : 0) + (a1 ? 1 : 0);
+    float2 acc[3][2];
 #pragma unroll
-    for (int a = 0; a < 3; a++) {
-        float h = axis_coord(p[a], b.plo[a], b.kp[a]);
-        const int u = min(max(__float2int_rd(h), 0), b.P - 2);
-        h = fminf(fmaxf(h, 0.f), (float)(b.P - 1));
-        h0[a] = u;
-        hf[a] = h - (float)u;
+    for (int k = 0; k < 3; k++) {
+        acc[k][0] = acc[k][1] = make_float2(0.f, 0.f);
+        pends[k] = gp[k] ? (pends[k] | cuts) >> j0 : 0u;
     }
-    const int64_t P = b.P;
+    for (int j = 0; j < len; j++) {
+        const float4 h = *reinterpret_cast<const float4 *>(t[j].hf);
+        const uint4 x = *reinterpret_cast<const uint4 *>(t[j].texel);
+        const float4 v = *reinterpret_cast<const float4 *>(t[j].gf + half);
+        const float u0 = fmaf(h.x, s1, c1), u1 = fmaf(h.y, s1, c1), v1 = fmaf(h.y, s2, c2), v2 = fmaf(h.z, s2, c2);
+        add_half(acc[0], v1 * u0, v);
+        add_half(acc[1], v2 * u0, v);
+        add_half(acc[2], v2 * u1, v);
+        if ((pends[0] >> j) & 1u) flush_half(gp[0] + 8 * (uint64_t)(x.x + off) + half, acc[0]);
+        if ((pends[1] >> j) & 1u) flush_half(gp[1] + 8 * (uint64_t)(x.y + off) + half, acc[1]);
+        if ((pends[2] >> j) & 1u) flush_half(gp[2] + 8 * (uint64_t)(x.z + off) + half, acc[2]);
+    }
+    __syncwarp();
+}
+
+// What the re-march of a ray carries from sample to sample: the transmittance
+// (uniform) and, in lane q < 7, the prefix sum of channel q of (C_d, F).
+struct BwdRay {
+    float T = 1.f, pre = 0.f;
+};
+
+// Re-march the warp's ray through one block and scatter its feature gradients.
+// gcf: dL/dC_d, dL/dF (uniform); total: the ray's (or the block's) final sum
+// of lane q's channel; Q: what else depends on the samples' transmittance.
+// Prefix and transmittance are taken in lattice order with the forward's
+// operations, so total - prefix is exactly what the forward added after the
+// sample.  Returns false when the ray ended early.
+template <int DT>
+__device__ __forceinline__ bool remarch_block(BwdScratch &bs, const BlockRec &b, const float o[3], const float d[3],
+                                              const float inv_d[3], float omax, const float gcf[7], float total,
+                                              float Q, float ert_eps, BwdRay &s, float *gg, float *const gp[3],
+                                              unsigned *err) {
+    const int lane = threadIdx.x & 31;
+    WarpScratch &ws = bs.w;
+    BrickCache bc;
+    return for_each_chunk(ws, b, o, d, inv_d, omax, err, [&](bool active, int n, const float p[3], const float g[3],
+                                                             float delta) {
+        float e = 1.f, sigma = 0.f, gdot = 0.f, c[7] = {0.f, 0.f, 0.f, 0.f, 0.f, 0.f, 0.f};
+        if (active) {
+            float2 f2[4];
+            accumulate_sample<DT>(b, p, g, f2, &bc);
+            const float f[8] = {f2[0].x, f2[0].y, f2[1].x, f2[1].y, f2[2].x, f2[2].y, f2[3].x, f2[3].y};
+            sigma = __expf(f[0]);
+            e = __expf(-sigma * delta);
 #pragma unroll
-    for (int pl = 0; pl < 3; pl++) {
-        if (!gp[pl]) continue;
-        const int ua = pl == 2 ? 1 : 0, va = pl == 0 ? 1 : 2;
-        const int64_t tb = (int64_t)h0[va] * P + h0[ua];
-        const float wu[2] = {1.f - hf[ua], hf[ua]}, wv[2] = {1.f - hf[va], hf[va]};
-#pragma unroll
-        for (int q = 0; q < 4; q++) {
-            const int du = q & 1, dv = q >> 1;
-            red_add8(gp[pl] + 8 * (tb + dv * P + du), wv[dv] * wu[du], gf);
+            for (int q = 0; q < 7; q++) {
+                c[q] = sigmoidf_fast(f[1 + q]);
+                gdot = fmaf(gcf[q], c[q], gdot);
+            }
         }
-    }
+#pragma unroll
+        for (int q = 0; q < 7; q++) ws.row[q][lane] = c[q];
+        ws.row[7][lane] = e;
+        __syncwarp();
+        float T = s.T;
+        if (lane < 8) {  // lane q < 7: total - prefix after every sample, in place; lane 7: T in front of it
+            float4 *x4 = reinterpret_cast<float4 *>(lane < 7 ? ws.row[lane] : bs.T);
+            const float4 *e4 = reinterpret_cast<const float4 *>(ws.row[7]);
+            float pre = s.pre;
+#pragma unroll
+            for (int k = 0; k < 8; k++) {
+                if (4 * k >= n) break;
+                const float4 ee = e4[k], xx = lane < 7 ? x4[k] : make_float4(0.f, 0.f, 0.f, 0.f);
+                const float Ts[4] = {T, T * ee.x, (T * ee.x) * ee.y, ((T * ee.x) * ee.y) * ee.z};
+                const float xv[4] = {xx.x, xx.y, xx.z, xx.w};
+                float w[4], out[4];
+                chunk_weights(ee, T, w);
+#pragma unroll
+                for (int j = 0; j < 4; j++) {
+                    pre = fmaf(w[j], xv[j], pre);
+                    out[j] = lane < 7 ? total - pre : Ts[j];
+                }
+                x4[k] = make_float4(out[0], out[1], out[2], out[3]);
+            }
+            s.pre = pre;
+        }
+        T = __shfl_sync(kFullMask, T, 0);
+        bool more = true;
+        int used = n;
+        if (T < ert_eps) {  // the ray ends in this chunk
+            more = false;
+            float Ts = s.T;
+            for (used = 0; used < n;) {
+                Ts *= ws.row[7][used++];
+                if (Ts < ert_eps) break;
+            }
+        }
+        s.T = T;
+        __syncwarp();
+        float gf[8];
+        {
+            const float Tb = bs.T[lane], wt = Tb * (1.f - e);
+            float sdot = Q;
+#pragma unroll
+            for (int q = 0; q < 7; q++) sdot = fmaf(gcf[q], ws.row[q][lane], sdot);
+            gf[0] = sigma * delta * (Tb * e * gdot - sdot);
+#pragma unroll
+            for (int q = 0; q < 7; q++) gf[1 + q] = wt * gcf[q] * c[q] * (1.f - c[q]);
+        }
+        scatter_chunk(b, bs.tap, used, p, g, gf, gg, gp);
+        return more;
+    });
 }
 
 // K7: deferred-MLP backward per ray; writes (dL/dC_d, dL/dF) of the ray to
@@ -198,73 +374,29 @@ __global__ void __launch_bounds__(kBwdThreads) k_mlp_backward(BwdArgs a) {
     }
 }
 
-// K6: re-march and scatter the feature gradients.
+// K6: re-march and scatter the feature gradients, one ray per warp.
 template <int DT>
-__global__ void __launch_bounds__(kBwdThreads, COW_BWD_MIN_BLOCKS) k_remarch_backward(BwdArgs a,
-                                                                                const __grid_constant__ RayRecs rr) {
-    const int64_t t = (int64_t)blockIdx.x * kBwdThreads + threadIdx.x;
-    if (t >= a.n_rays) return;
-    const int64_t r = a.ray_perm ? (int64_t)__ldg(a.ray_perm + t) : t;
-    float o[3], d[3], Cf[3], Ff[4], gC[3], gF[4];
-#pragma unroll
-    for (int c = 0; c < 3; c++) {
-        o[c] = __ldg(a.ray_o + 3 * r + c);
-        d[c] = __ldg(a.ray_d + 3 * r + c);
-        Cf[c] = __ldg(a.aux + 8 * r + c);
-        gC[c] = __ldg(a.gcf + 8 * r + c);
-    }
-#pragma unroll
-    for (int c = 0; c < 4; c++) {
-        Ff[c] = __ldg(a.aux + 8 * r + 3 + c);
-        gF[c] = __ldg(a.gcf + 8 * r + 3 + c);
-    }
-    int order[kMaxRayIds];
-    const int n = sort_blocks_for_ray(rr, o, order);
-    float inv_d[3], omax;
+__global__ void __launch_bounds__(kBwdThreads, COW_BWD_MIN_BLOCKS) k_remarch_backward(
+    const __grid_constant__ BwdArgs a, const __grid_constant__ RayRecs rr) {
+    __shared__ BwdScratch s_bs[kBwdWarps];
+    BwdScratch &bs = s_bs[threadIdx.x >> 5];
+    const int lane = threadIdx.x & 31;
+    float o[3], d[3], inv_d[3], omax;
+    const int64_t r = load_ray_warp(a, o, d);
+    if (r < 0) return;
     ray_setup(d, o, inv_d, omax);
-    float T = 1.f, PC[3] = {0.f, 0.f, 0.f}, PF[4] = {0.f, 0.f, 0.f, 0.f};
-    for (int k = 0; k < n; k++) {
-        const int id = rr.id[order[k]];
-        const BlockRec &b = rr.r[order[k]];
-        float *gg = a.grad_grid[id];
+    float gcf[7];
+#pragma unroll
+    for (int q = 0; q < 7; q++) gcf[q] = __ldg(a.gcf + 8 * r + q);
+    const float total = __ldg(a.aux + 8 * r + (lane & 7));
+    const int n = sort_blocks_warp(bs.w, rr, o);
+    BwdRay s;
+    for_each_hit(n, [&](int k) -> const BlockRec & { return rr.r[bs.w.ord[k]]; }, o, d, inv_d, [&](int k) {
+        const int id = rr.id[bs.w.ord[k]];
         float *const gp[3] = {a.grad_planes[3 * id], a.grad_planes[3 * id + 1], a.grad_planes[3 * id + 2]};
-        BrickCache bc;
-        const bool more = for_each_sample(b, o, d, inv_d, omax, a.err, [&](const float p[3], const float g[3],
-                                                                           float delta) {
-            float2 f2[4];
-            accumulate_sample<DT>(b, p, g, f2, &bc);
-            const float f[8] = {f2[0].x, f2[0].y, f2[1].x, f2[1].y, f2[2].x, f2[2].y, f2[3].x, f2[3].y};
-            const float sigma = __expf(f[0]);
-            const float e = __expf(-sigma * delta);
-            const float wt = T * (1.f - e);
-            float c[7];
-#pragma unroll
-            for (int q = 0; q < 7; q++) c[q] = sigmoidf_fast(f[1 + q]);
-            float gdot = 0.f, sdot = 0.f;
-#pragma unroll
-            for (int q = 0; q < 3; q++) {
-                PC[q] = fmaf(wt, c[q], PC[q]);
-                gdot = fmaf(gC[q], c[q], gdot);
-                sdot = fmaf(gC[q], Cf[q] - PC[q], sdot);
-            }
-#pragma unroll
-            for (int q = 0; q < 4; q++) {
-                PF[q] = fmaf(wt, c[3 + q], PF[q]);
-                gdot = fmaf(gF[q], c[3 + q], gdot);
-                sdot = fmaf(gF[q], Ff[q] - PF[q], sdot);
-            }
-            float gf[8];
-            gf[0] = sigma * delta * (T * e * gdot - sdot);
-#pragma unroll
-            for (int q = 0; q < 3; q++) gf[1 + q] = wt * gC[q] * c[q] * (1.f - c[q]);
-#pragma unroll
-            for (int q = 0; q < 4; q++) gf[4 + q] = wt * gF[q] * c[3 + q] * (1.f - c[3 + q]);
-            scatter_taps(b, gg, gp, p, g, gf);
-            T *= e;
-            return !(T < a.ert_eps);
-        });
-        if (!more) break;
-    }
+        return remarch_block<DT>(bs, rr.r[bs.w.ord[k]], o, d, inv_d, omax, gcf, total, 0.f, a.ert_eps, s,
+                                 a.grad_grid[id], gp, a.err);
+    });
 }
 
 // ---------------------------------------------------------------------------
@@ -495,33 +627,28 @@ __device__ __forceinline__ float bm_input(int i, const float ck[7], const float 
 
 // P1
 template <int DT>
-__global__ void __launch_bounds__(kBwdThreads) k_bm_pass1(BmBwdArgs a, const __grid_constant__ RayRecs rr) {
-    const int64_t t = (int64_t)blockIdx.x * kBwdThreads + threadIdx.x;
-    if (t >= a.n_rays) return;
-    const int64_t r = a.ray_perm ? (int64_t)__ldg(a.ray_perm + t) : t;
-    float o[3], d[3];
-#pragma unroll
-    for (int c = 0; c < 3; c++) {
-        o[c] = __ldg(a.ray_o + 3 * r + c);
-        d[c] = __ldg(a.ray_d + 3 * r + c);
-    }
-    int order[kMaxRayIds];
-    const int n = sort_blocks_for_ray(rr, o, order);
-    float inv_d[3], omax;
+__global__ void __launch_bounds__(kBwdThreads) k_bm_pass1(const __grid_constant__ BmBwdArgs a,
+                                                          const __grid_constant__ RayRecs rr) {
+    __shared__ WarpScratch s_ws[kBwdWarps];
+    WarpScratch &ws = s_ws[threadIdx.x >> 5];
+    const int lane = threadIdx.x & 31;
+    float o[3], d[3], inv_d[3], omax;
+    const int64_t r = load_ray_warp(a, o, d);
+    if (r < 0) return;
     ray_setup(d, o, inv_d, omax);
+    const int n = sort_blocks_warp(ws, rr, o);
+    float *S = a.S + 8 * r * a.n_ids;
+    for (int k = lane; k < n; k += 32) S[8 * k + 7] = -1.f;  // no occupied sample
+    __syncwarp();
     float B = 1.f;
-    for (int k = 0; k < n; k++) {
-        RayState sb = {{0.f, 0.f, 0.f}, {0.f, 0.f, 0.f, 0.f}, 1.f, 0, false};
-        march_block<DT>(rr.r[order[k]], o, d, inv_d, omax, 0.f, sb, a.err);
-        float4 *e = reinterpret_cast<float4 *>(a.S + 8 * (r * a.n_ids + order[k]));
-        if (sb.nsamp == 0) {
-            e[1] = make_float4(0.f, 0.f, 0.f, -1.f);
-            continue;
-        }
-        e[0] = make_float4(sb.Cd[0], sb.Cd[1], sb.Cd[2], sb.F[0]);
-        e[1] = make_float4(sb.F[1], sb.F[2], sb.F[3], B);
+    for_each_hit(n, [&](int k) -> const BlockRec & { return rr.r[ws.ord[k]]; }, o, d, inv_d, [&](int k) {
+        WarpRay sb;
+        march_block_warp<DT>(ws, rr.r[ws.ord[k]], o, d, inv_d, omax, 0.f, sb, a.err);
+        if (sb.nsamp == 0) return true;
+        if (lane < 8) S[8 * ws.ord[k] + lane] = lane < 7 ? sb.acc : B;
         B *= sb.T;
-    }
+        return true;
+    });
 }
 
 // A weight-gradient term summed over the warp's 32 rays, then one reduction.
@@ -673,86 +800,39 @@ __global__ void __launch_bounds__(kBwdThreads) k_bm_mlp(BmBwdArgs a, const __gri
     go[1] = make_float4(gx[4], gx[5], gx[6], xg);
 }
 
-// P3
+// P3, one ray per warp
 template <int DT>
-__global__ void __launch_bounds__(kBwdThreads, COW_BWD_MIN_BLOCKS) k_bm_remarch(BmBwdArgs a,
+__global__ void __launch_bounds__(kBwdThreads, COW_BWD_MIN_BLOCKS) k_bm_remarch(const __grid_constant__ BmBwdArgs a,
                                                                           const __grid_constant__ RayRecs rr) {
-    const int64_t t = (int64_t)blockIdx.x * kBwdThreads + threadIdx.x;
-    if (t >= a.n_rays) return;
-    const int64_t r = a.ray_perm ? (int64_t)__ldg(a.ray_perm + t) : t;
-    float o[3], d[3];
-#pragma unroll
-    for (int c = 0; c < 3; c++) {
-        o[c] = __ldg(a.ray_o + 3 * r + c);
-        d[c] = __ldg(a.ray_d + 3 * r + c);
-    }
+    __shared__ BwdScratch s_bs[kBwdWarps];
+    BwdScratch &bs = s_bs[threadIdx.x >> 5];
+    const int lane = threadIdx.x & 31;
+    float o[3], d[3], inv_d[3], omax;
+    const int64_t r = load_ray_warp(a, o, d);
+    if (r < 0) return;
+    ray_setup(d, o, inv_d, omax);
     const float *S = a.S + 8 * r * a.n_ids, *G = a.G + 8 * r * a.n_ids;
     float Qtot = 0.f;  // sum_k B_k dL/dC . X_k
     for (int k = 0; k < a.n_ids; k++) {
         const float B = __ldg(S + 8 * k + 7);
         if (B >= 0.f) Qtot = fmaf(B, __ldg(G + 8 * k + 7), Qtot);
     }
-    int order[kMaxRayIds];
-    const int n = sort_blocks_for_ray(rr, o, order);
-    float inv_d[3], omax;
-    ray_setup(d, o, inv_d, omax);
+    const int n = sort_blocks_warp(bs.w, rr, o);
     float P = 0.f;
     for (int k = 0; k < n; k++) {
-        const int idx = order[k];
+        const int idx = bs.w.ord[k];
         const float B = __ldg(S + 8 * idx + 7);
         if (B < 0.f) continue;  // no occupied sample: no part in Eq. 5
-        float Cf[3], Ff[4], gC[3], gF[4];
+        float gcf[7];
 #pragma unroll
-        for (int c = 0; c < 3; c++) {
-            Cf[c] = __ldg(S + 8 * idx + c);
-            gC[c] = __ldg(G + 8 * idx + c);
-        }
-#pragma unroll
-        for (int c = 0; c < 4; c++) {
-            Ff[c] = __ldg(S + 8 * idx + 3 + c);
-            gF[c] = __ldg(G + 8 * idx + 3 + c);
-        }
+        for (int q = 0; q < 7; q++) gcf[q] = __ldg(G + 8 * idx + q);
         P = fmaf(B, __ldg(G + 8 * idx + 7), P);
-        const float Q = Qtot - P;  // the blocks behind this one
         const int id = rr.id[idx];
-        const BlockRec &b = rr.r[idx];
-        float *gg = a.grad_grid[id];
         float *const gp[3] = {a.grad_planes[3 * id], a.grad_planes[3 * id + 1], a.grad_planes[3 * id + 2]};
-        float T = 1.f, PC[3] = {0.f, 0.f, 0.f}, PF[4] = {0.f, 0.f, 0.f, 0.f};
-        BrickCache bc;
-        for_each_sample(b, o, d, inv_d, omax, a.err, [&](const float p[3], const float g[3], float delta) {
-            float2 f2[4];
-            accumulate_sample<DT>(b, p, g, f2, &bc);
-            const float f[8] = {f2[0].x, f2[0].y, f2[1].x, f2[1].y, f2[2].x, f2[2].y, f2[3].x, f2[3].y};
-            const float sigma = __expf(f[0]);
-            const float e = __expf(-sigma * delta);
-            const float wt = T * (1.f - e);
-            float c[7];
-#pragma unroll
-            for (int q = 0; q < 7; q++) c[q] = sigmoidf_fast(f[1 + q]);
-            float gdot = 0.f, sdot = Q;
-#pragma unroll
-            for (int q = 0; q < 3; q++) {
-                PC[q] = fmaf(wt, c[q], PC[q]);
-                gdot = fmaf(gC[q], c[q], gdot);
-                sdot = fmaf(gC[q], Cf[q] - PC[q], sdot);
-            }
-#pragma unroll
-            for (int q = 0; q < 4; q++) {
-                PF[q] = fmaf(wt, c[3 + q], PF[q]);
-                gdot = fmaf(gF[q], c[3 + q], gdot);
-                sdot = fmaf(gF[q], Ff[q] - PF[q], sdot);
-            }
-            float gf[8];
-            gf[0] = sigma * delta * (T * e * gdot - sdot);
-#pragma unroll
-            for (int q = 0; q < 3; q++) gf[1 + q] = wt * gC[q] * c[q] * (1.f - c[q]);
-#pragma unroll
-            for (int q = 0; q < 4; q++) gf[4 + q] = wt * gF[q] * c[3 + q] * (1.f - c[3 + q]);
-            scatter_taps(b, gg, gp, p, g, gf);
-            T *= e;
-            return true;
-        });
+        BwdRay s;
+        // Q: the blocks behind this one
+        remarch_block<DT>(bs, rr.r[idx], o, d, inv_d, omax, gcf, __ldg(S + 8 * idx + (lane & 7)), Qtot - P, 0.f, s,
+                          a.grad_grid[id], gp, a.err);
     }
 }
 
@@ -763,13 +843,14 @@ int backward_rows(int64_t n_rays) { return (int)((n_rays + kBwdThreads - 1) / kB
 cudaError_t launch_backward_rays(const BwdArgs &a, const RayRecs &rr, cudaStream_t st) {
     if (a.n_rays <= 0) return cudaSuccess;
     const int nb = backward_rows(a.n_rays);
+    const unsigned nw = (unsigned)((a.n_rays + kBwdWarps - 1) / kBwdWarps);  // one ray per warp
     k_mlp_backward<<<nb, kBwdThreads, 0, st>>>(a);
     cudaError_t e = cudaGetLastError();
     if (e != cudaSuccess) return e;
     k_reduce_rows<<<(kMlpParams + 127) / 128, 128, 0, st>>>(a.partials, nb, a.grad_mlp);
     {
         const cudaError_t e_ = dispatch_dt(a.dtype, [&](auto D) {
-            k_remarch_backward<decltype(D)::value><<<nb, kBwdThreads, 0, st>>>(a, rr);
+            k_remarch_backward<decltype(D)::value><<<nw, kBwdThreads, 0, st>>>(a, rr);
             return cudaSuccess;
         });
         if (e_ != cudaSuccess) return e_;
@@ -779,11 +860,11 @@ cudaError_t launch_backward_rays(const BwdArgs &a, const RayRecs &rr, cudaStream
 
 cudaError_t launch_backward_block_mlps(const BmBwdArgs &a, const RayRecs &rr, cudaStream_t st) {
     if (a.n_rays <= 0) return cudaSuccess;
-    const int nb = backward_rows(a.n_rays);
+    const unsigned nw = (unsigned)((a.n_rays + kBwdWarps - 1) / kBwdWarps);  // one ray per warp
     const int64_t padded = ((a.n_rays + 31) & ~(int64_t)31) * a.n_ids;  // k_bm_mlp's threads
     if (!a.have_state) {
         const cudaError_t e_ = dispatch_dt(a.dtype, [&](auto D) {
-            k_bm_pass1<decltype(D)::value><<<nb, kBwdThreads, 0, st>>>(a, rr);
+            k_bm_pass1<decltype(D)::value><<<nw, kBwdThreads, 0, st>>>(a, rr);
             return cudaSuccess;
         });
         if (e_ != cudaSuccess) return e_;
@@ -794,7 +875,7 @@ cudaError_t launch_backward_block_mlps(const BmBwdArgs &a, const RayRecs &rr, cu
     if ((e = cudaGetLastError()) != cudaSuccess) return e;
     {
         const cudaError_t e_ = dispatch_dt(a.dtype, [&](auto D) {
-            k_bm_remarch<decltype(D)::value><<<nb, kBwdThreads, 0, st>>>(a, rr);
+            k_bm_remarch<decltype(D)::value><<<nw, kBwdThreads, 0, st>>>(a, rr);
             return cudaSuccess;
         });
         if (e_ != cudaSuccess) return e_;

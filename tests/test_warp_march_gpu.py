@@ -10,6 +10,7 @@ import torch
 
 import oracle
 from paper_2312_16457_gb300 import cow, synth
+from gradcheck import assert_grad
 
 pytestmark = pytest.mark.gpu
 SAME = 2e-6
@@ -106,4 +107,52 @@ def test_block_order_beyond_a_warp(n_ids):
     hit = bt >= 0
     assert torch.equal(hit.any(1), ns > 0) and float((part[..., 7] - torch.where(hit, bt, 1.0)).abs().max()) <= SAME
     assert float((torch.where(hit, bt, 1.0).prod(1) - aux[:, 7]).abs().max()) <= 1e-5
+    ctx.close()
+
+
+@pytest.mark.parametrize("form", ["fp32", "bf16", "fp16 unbounded"])
+def test_backward_edges(form):
+    """The cooperative scatter at partial chunks and CTAs, odd resolutions and
+    contracted blocks: 300 rays at once against the oracle's gradient, and the
+    same rays in calls of 1, 5, 33 and 261 against that up to the order of the
+    FP32 reductions (1e-5 of each array's largest entry); arrays that are not
+    asked for stay out of it."""
+    storage, *opt = form.split()
+    n = 300
+    sc, _, mlp = _scene("unbounded" in opt)
+    o, d = synth.random_rays(n, 12, sc.box_lo, sc.box_hi)
+    if "unbounded" in opt:
+        o = torch.tensor([0.25, -0.4, 0.3]).expand(n, 3).contiguous()
+    g = np.random.default_rng(6).normal(size=(n, 3)).astype(np.float32)
+    ctx = cow.Context(sc, storage)
+    ids = list(range(4))
+    oc, dc, gc, mc = o.cuda(), d.cuda(), torch.from_numpy(g).cuda(), torch.from_numpy(mlp).cuda()
+    _, aux, _ = ctx.render_rays(oc, dc, ids, mc)
+    res = []
+    for cuts in ((0, n), (0, 1, 6, 39, n)):
+        gg = [torch.zeros(b.grid.shape, device="cuda") for b in sc.blocks]
+        gp = [[torch.zeros(p.shape, device="cuda") for p in b.planes] for b in sc.blocks]
+        gm = torch.zeros(499, device="cuda")
+        ga, pa = list(gg), [list(p) for p in gp]
+        if len(cuts) > 2:  # without block 1's grid and block 2's xz plane
+            ga[1], pa[2][1] = None, None
+        for a, b in zip(cuts, cuts[1:]):
+            ctx.render_backward(oc[a:b], dc[a:b], ids, mc, aux[a:b], gc[a:b], ga, pa, gm)
+        ctx.sync_check()
+        res.append((gg, gp, gm))
+    og, op, om = oracle.render_rays_grad(
+        oracle.OracleScene(sc, values="master" if storage == "fp32" else storage), ids, o, d, mlp, g)
+    (gg, gp, gm), (sg, sp, sm) = res
+    assert_grad(gm, om, "mlp")
+
+    def close(x, y):
+        assert float((x - y).abs().max()) <= 1e-5 * float(y.abs().max())
+
+    close(sm, gm)
+    for b in range(4):
+        assert_grad(gg[b], og[b], f"grid {b}")
+        close(sg[b], gg[b] * (b != 1))
+        for k in range(3):
+            assert_grad(gp[b][k], op[b][k], f"plane {b} {k}")
+            close(sp[b][k], gp[b][k] * ((b, k) != (2, 1)))
     ctx.close()
