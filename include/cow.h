@@ -660,16 +660,16 @@ cow_status cow_set_schedule(cow_ctx *ctx, int32_t schedule);
  * cow_render_rays_block_t, cow_render_partials, cow_render_backward,
  * cow_render_backward_block_mlps, cow_opacity_loss).  COW_RAY_ORDER_COHERENT (default): a
  * batch of at least 8192 rays is marched in a coherent order -- rays grouped
- * by the cell of their entry into the call's blocks' bounding box (8 x 8 x 8)
- * and of their direction (8 x 8 x 8), by a counting sort on the device -- so
- * that the rays on the chip at one time gather neighbouring texels and share
- * them in L2 (measured on 2^20 random rays over 2x2 blocks of 128^3 / 512^2
- * FP32 features: forward 39.9 -> 31.1 ms).  COW_RAY_ORDER_GIVEN: warp t marches
- * ray t.  cow_render_rays of 2^17 rays or more that are mostly alike their
- * neighbours (a camera's rays) are marched one ray per thread in the given order.  Outputs are written at each ray's own index either way and each
- * ray's values are the same; gradient sums change only by the order of their
- * FP32 reductions.  The order costs a key pass, a scan and a scatter (about
- * 12 bytes a ray and 1 MiB of context scratch).  Errors: INVALID_ARG. */
+ * by the cells in which they enter and leave the call's blocks' bounding box,
+ * by a counting sort on the device -- so that the rays on the chip at one time
+ * gather neighbouring texels and share them in L2 (measured on 2^20 random rays
+ * over 2x2 blocks of 128^3 / 512^2 FP32 features: forward 39.9 -> 28.3 ms).
+ * COW_RAY_ORDER_GIVEN: warp t marches ray t.  cow_render_rays of 2^17 rays or
+ * more that are mostly alike their neighbours (a camera's rays) are marched one
+ * ray per thread in the given order.  Outputs are written at each ray's own
+ * index either way and each ray's values are the same; gradient sums change
+ * only by the order of their FP32 reductions.  The order costs a key pass, a scan and a scatter (about
+ * 12 bytes a ray and 4 MiB of context scratch).  Errors: INVALID_ARG. */
 #define COW_RAY_ORDER_GIVEN 0
 #define COW_RAY_ORDER_COHERENT 1
 cow_status cow_set_ray_order(cow_ctx *ctx, int32_t mode);

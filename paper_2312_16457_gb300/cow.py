@@ -499,7 +499,7 @@ class Context:
 
     def set_ray_order(self, mode: str):
         """Processing order of ray batches: "coherent" (default; rays grouped by
-        entry cell and direction) or "given"."""
+        entry and exit cell) or "given"."""
         _check(lib().cow_set_ray_order(self._ctx, self.RAY_ORDERS[mode]))
 
     def set_schedule(self, name: str):

@@ -55,13 +55,13 @@ struct ParamRecs;
 cudaError_t launch_march_views(const MarchArgs &a, int n_tiles, int schedule, cudaStream_t st,
                                const ParamRecs *pr = nullptr);
 cudaError_t launch_march_rays(const MarchArgs &a, const RayRecs &rr, cudaStream_t st);
-// A coherent order of a ray batch (ray_order.cu): perm[t] = the ray thread t
-// marches, grouping rays by the cell of their entry into the box [lo, hi]
-// and of their direction.  keys: n scratch words; hist: kRayOrderHistWords
+// A coherent order of a ray batch (ray_order.cu): perm[t] = the ray warp t
+// marches, grouping rays by the cells of their entry into the box [lo, hi]
+// and their exit from it.  keys: n scratch words; hist: kRayOrderHistWords
 // words (the bins; at kRayOrderAlike the count of rays whose key is the next
 // ray's; the totals of the scan's blocks of 1024 bins).  perm may be null: the
 // count alone.
-constexpr int kRayOrderKeyBits = 18;
+constexpr int kRayOrderKeyBits = 20;
 constexpr int kRayOrderBins = 1 << kRayOrderKeyBits;
 constexpr int kRayOrderAlike = kRayOrderBins;
 constexpr int kRayOrderHistWords = kRayOrderBins + 32 + kRayOrderBins / 1024;
