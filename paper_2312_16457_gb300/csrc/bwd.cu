@@ -27,6 +27,8 @@
 // The CTA's MLP weight gradient (499 sums over its 128 rays) goes to a
 // per-CTA scratch row; a second kernel adds the rows in a fixed order, so the
 // MLP gradient does not depend on scheduling.
+#include <algorithm>
+
 #include "cow_common.cuh"
 #include "cow_kernels.h"
 #include "march_core.cuh"
@@ -43,9 +45,7 @@ namespace {
 #endif
 
 #ifndef COW_REG_MIN_BLOCKS
-// the same for the opacity regulariser's double march: 2 CTAs per SM took a
-// regularised fit step from ~496 to ~473 ms
-#define COW_REG_MIN_BLOCKS 2
+#define COW_REG_MIN_BLOCKS 4  // 6 and 8 measured the same
 #endif
 
 constexpr int kBwdThreads = kBwdCtaThreads;
@@ -71,8 +71,9 @@ struct alignas(16) TapRec {
     uint32_t base_lo;   // the voxel's first vertex
     float hf[3];        // places inside the texel cells along x, y, z
     uint32_t base_hi;
-    uint32_t texel[4];  // first texel of the xy, xz, yz footprints; unused
-    float gf[8];
+    uint32_t texel[3];  // first texel of the xy, xz, yz footprints
+    float g0;           // gradient of channel 0
+    float gf[8];        // of all eight
 };
 
 // Shared scratch of one warp of the re-march.
@@ -101,16 +102,12 @@ __device__ __forceinline__ void flush_half(float *dst, float2 acc[2]) {
     acc[0] = acc[1] = make_float2(0.f, 0.f);
 }
 
-// Scatter a chunk of n samples (lane j < n holds sample j's point and gradient
-// gf) to the taps of their lookups, as a warp: a lane has one tap and one half
-// of its eight channels, so the lanes of one reduction cover whole 64-byte
-// vertex or texel pairs (the L2 takes 64-byte groups of float4 reductions 1.6
-// times as fast as scattered ones: 330 against 205 G/s into 32 MiB, 147 against
-// 46 G/s into 256 MiB), and it walks its samples in ray order, adding up what
-// goes to one voxel or texel cell before it issues the reduction (a lattice
-// step is about a quarter of a voxel, so a voxel takes some 2.5 samples).
-__device__ __forceinline__ void scatter_chunk(const BlockRec &b, TapRec *tap, int n, const float p[3],
-                                              const float g[3], const float gf[8], float *gg, float *const gp[3]) {
+// Put lane j's sample (j < n; point p, grid coordinate g, gradient gf) into
+// tap[j]; ends: where the chunk's runs of samples in one voxel end, pends[k]:
+// in one texel cell of plane k.
+template <int NCH>
+__device__ __forceinline__ void make_taps(const BlockRec &b, TapRec *tap, int n, const float p[3], const float g[3],
+                                          const float gf[NCH], unsigned &ends, unsigned pends[3]) {
     const int lane = threadIdx.x & 31;
     uint64_t base = 0;
     uint32_t tx[3] = {0, 0, 0};
@@ -133,19 +130,35 @@ __device__ __forceinline__ void scatter_chunk(const BlockRec &b, TapRec *tap, in
         float4 *o = reinterpret_cast<float4 *>(tap + lane);
         o[0] = make_float4(fr[0], fr[1], fr[2], __uint_as_float((uint32_t)base));
         o[1] = make_float4(hf[0], hf[1], hf[2], __uint_as_float((uint32_t)(base >> 32)));
-        o[2] = make_float4(__uint_as_float(tx[0]), __uint_as_float(tx[1]), __uint_as_float(tx[2]), 0.f);
-        o[3] = make_float4(gf[0], gf[1], gf[2], gf[3]);
-        o[4] = make_float4(gf[4], gf[5], gf[6], gf[7]);
+        o[2] = make_float4(__uint_as_float(tx[0]), __uint_as_float(tx[1]), __uint_as_float(tx[2]), gf[0]);
+        if constexpr (NCH == 8) {
+            o[3] = make_float4(gf[0], gf[1], gf[2], gf[3]);
+            o[4] = make_float4(gf[4], gf[5], gf[6], gf[7]);
+        }
     }
     const uint64_t pbase = __shfl_up_sync(kFullMask, base, 1);
-    unsigned ends = run_ends(pbase == base && lane > 0, n);
-    unsigned pends[3];
+    ends = run_ends(pbase == base && lane > 0, n);
 #pragma unroll
     for (int k = 0; k < 3; k++) {
         const uint32_t ptx = __shfl_up_sync(kFullMask, tx[k], 1);
         pends[k] = run_ends(ptx == tx[k] && lane > 0, n);
     }
     __syncwarp();
+}
+
+// Scatter a chunk of n samples (lane j < n holds sample j's point and gradient
+// gf) to the taps of their lookups, as a warp: a lane has one tap and one half
+// of its eight channels, so the lanes of one reduction cover whole 64-byte
+// vertex or texel pairs (the L2 takes 64-byte groups of float4 reductions 1.6
+// times as fast as scattered ones: 330 against 205 G/s into 32 MiB, 147 against
+// 46 G/s into 256 MiB), and it walks its samples in ray order, adding up what
+// goes to one voxel or texel cell before it issues the reduction (a lattice
+// step is about a quarter of a voxel, so a voxel takes some 2.5 samples).
+__device__ __forceinline__ void scatter_chunk(const BlockRec &b, TapRec *tap, int n, const float p[3],
+                                              const float g[3], const float gf[8], float *gg, float *const gp[3]) {
+    const int lane = threadIdx.x & 31;
+    unsigned ends, pends[3];
+    make_taps<8>(b, tap, n, p, g, gf, ends, pends);
     // place q (0 or 1) of an axis: weight 1 - f or f, as s f + c
     const float s1 = (lane & 2) ? 1.f : -1.f, c1 = (lane & 2) ? 0.f : 1.f;
     const float s2 = (lane & 4) ? 1.f : -1.f, c2 = (lane & 4) ? 0.f : 1.f;
@@ -191,6 +204,75 @@ __device__ __forceinline__ void scatter_chunk(const BlockRec &b, TapRec *tap, in
         if ((pends[0] >> j) & 1u) flush_half(gp[0] + 8 * (uint64_t)(x.x + off) + half, acc[0]);
         if ((pends[1] >> j) & 1u) flush_half(gp[1] + 8 * (uint64_t)(x.y + off) + half, acc[1]);
         if ((pends[2] >> j) & 1u) flush_half(gp[2] + 8 * (uint64_t)(x.z + off) + half, acc[2]);
+    }
+    __syncwarp();
+}
+
+// The same for the density channel alone: 8 lanes a run, one vertex each, then
+// one texel of the xy and xz planes each; 4 lanes a run for the yz plane.
+__device__ __forceinline__ void scatter_density_chunk(const BlockRec &b, TapRec *tap, int n, const float p[3],
+                                                      const float g[3], float g0, float *gg, float *const gp[3]) {
+    const int lane = threadIdx.x & 31;
+    unsigned ends, pends[3];
+    make_taps<1>(b, tap, n, p, g, &g0, ends, pends);
+    const bool a0 = lane & 1, a1 = lane & 2, a2 = lane & 4;
+    const float s0 = a0 ? 1.f : -1.f, c0 = a0 ? 0.f : 1.f, s1 = a1 ? 1.f : -1.f, c1 = a1 ? 0.f : 1.f;
+    const unsigned all = kFullMask >> (32 - n);
+    {
+        const int len = (n + 3) >> 2, j0 = (lane >> 3) * len;
+        const unsigned cuts = ((1u << (len - 1)) | (1u << (2 * len - 1)) | (1u << (3 * len - 1))) & all;
+        const TapRec *t = tap + j0;
+        if (gg) {
+            const float s2 = a2 ? 1.f : -1.f, c2 = a2 ? 0.f : 1.f;
+            const int64_t R = b.R;
+            float *const dst = gg + 8 * (((a2 ? R : 0) + (a1 ? 1 : 0)) * R + (a0 ? 1 : 0));
+            const unsigned mine = (ends | cuts) >> j0;
+            float acc = 0.f;
+#pragma unroll 2
+            for (int j = 0; j < len; j++) {
+                const float4 f = *reinterpret_cast<const float4 *>(t[j].fr);
+                acc = fmaf((fmaf(f.y, s1, c1) * fmaf(f.z, s2, c2)) * fmaf(f.x, s0, c0), t[j].g0, acc);
+                if ((mine >> j) & 1u) {
+                    red_add1(dst + 8 * ((uint64_t)t[j].base_hi << 32 | __float_as_uint(f.w)), acc);
+                    acc = 0.f;
+                }
+            }
+        }
+        // lanes with bit 2: the xz plane, the others: the xy plane
+        if (float *const gq = a2 ? gp[1] : gp[0]) {
+            const unsigned mine = ((a2 ? pends[1] : pends[0]) | cuts) >> j0;
+            const uint32_t off = (a1 ? b.P : 0) + (a0 ? 1 : 0);
+            float acc = 0.f;
+#pragma unroll 2
+            for (int j = 0; j < len; j++) {
+                const float4 h = *reinterpret_cast<const float4 *>(t[j].hf);
+                const float4 x = *reinterpret_cast<const float4 *>(t[j].texel);
+                acc = fmaf(fmaf(a2 ? h.z : h.y, s1, c1) * fmaf(h.x, s0, c0), x.w, acc);
+                if ((mine >> j) & 1u) {
+                    red_add1(gq + 8 * (uint64_t)(__float_as_uint(a2 ? x.y : x.x) + off), acc);
+                    acc = 0.f;
+                }
+            }
+        }
+    }
+    if (gp[2]) {
+        const int len = (n + 7) >> 3, j0 = (lane >> 2) * len;
+        unsigned cuts = 0;
+        for (int k = 1; k < 8; k++) cuts |= 1u << (k * len - 1);
+        const unsigned mine = j0 < n ? (pends[2] | (cuts & all)) >> j0 : 0u;
+        const TapRec *t = tap + min(j0, n - 1);
+        const uint32_t off = (a1 ? b.P : 0) + (a0 ? 1 : 0);
+        float acc = 0.f;
+        for (int j = 0; j < len; j++) {
+            if (j0 + j >= n) break;
+            const float4 h = *reinterpret_cast<const float4 *>(t[j].hf);
+            const float4 x = *reinterpret_cast<const float4 *>(t[j].texel);
+            acc = fmaf(fmaf(h.z, s1, c1) * fmaf(h.y, s0, c0), x.w, acc);
+            if ((mine >> j) & 1u) {
+                red_add1(gp[2] + 8 * (uint64_t)(__float_as_uint(x.z) + off), acc);
+                acc = 0.f;
+            }
+        }
     }
     __syncwarp();
 }
@@ -382,7 +464,7 @@ __global__ void __launch_bounds__(kBwdThreads, COW_BWD_MIN_BLOCKS) k_remarch_bac
     BwdScratch &bs = s_bs[threadIdx.x >> 5];
     const int lane = threadIdx.x & 31;
     float o[3], d[3], inv_d[3], omax;
-    const int64_t r = load_ray_warp(a, o, d);
+    const int64_t r = load_ray_warp(a, first_ray(), o, d);
     if (r < 0) return;
     ray_setup(d, o, inv_d, omax);
     float gcf[7];
@@ -410,8 +492,9 @@ __global__ void __launch_bounds__(kBwdThreads, COW_BWD_MIN_BLOCKS) k_remarch_bac
 //     d alpha^k / d f0_i = sigma_i delta (1 - alpha^k).  The block is marched
 //     once for alpha^k -- or alpha^k comes from the forward's in-block
 //     transmittance -- and once to scatter.
-// Gradients reach the density channel only: 20 scalar atomics per point or
-// sample (8 grid vertices, 4 texels of each plane).
+// Gradients reach the density channel only: 20 scalar reductions per point or
+// sample (8 grid vertices, 4 texels of each plane), in the opacity term added
+// up per voxel and texel cell first.
 
 __device__ __forceinline__ void scatter_ch0(const BlockRec &b, float *gg, float *const gp[3], const float p[3],
                                             const float g[3], float g0) {
@@ -458,26 +541,26 @@ __device__ __forceinline__ void scatter_ch0(const BlockRec &b, float *gg, float 
     }
 }
 
-// sum of v over the CTA, added to *loss by one thread
-__device__ __forceinline__ void add_loss(float v, float *loss) {
+// sum of v over the CTA, in thread 0
+__device__ __forceinline__ float cta_sum(float v) {
     __shared__ float s_part[32];
 #pragma unroll
     for (int off = 16; off > 0; off >>= 1) v += __shfl_xor_sync(0xffffffffu, v, off);
     if ((threadIdx.x & 31) == 0) s_part[threadIdx.x >> 5] = v;
     __syncthreads();
     if (threadIdx.x < 32) {
-        float w = threadIdx.x < (blockDim.x >> 5) ? s_part[threadIdx.x] : 0.f;
+        v = threadIdx.x < (blockDim.x >> 5) ? s_part[threadIdx.x] : 0.f;
 #pragma unroll
-        for (int off = 16; off > 0; off >>= 1) w += __shfl_xor_sync(0xffffffffu, w, off);
-        if (threadIdx.x == 0 && loss) atomicAdd(loss, w);
+        for (int off = 16; off > 0; off >>= 1) v += __shfl_xor_sync(0xffffffffu, v, off);
     }
+    return v;
 }
 
 template <int DT>
 __global__ void __launch_bounds__(kBwdThreads) k_sparsity(RegArgs a, const __grid_constant__ RayRecs rr) {
     const int64_t r = (int64_t)blockIdx.x * kBwdThreads + threadIdx.x;
     float term = 0.f;
-    if (r < a.n) {
+    if (r < a.n_rays) {
         const float p[3] = {__ldg(a.pts + 3 * r), __ldg(a.pts + 3 * r + 1), __ldg(a.pts + 3 * r + 2)};
         int pos = -1;
         for (int k = 0; k < rr.n && pos < 0; k++) {
@@ -493,7 +576,7 @@ __global__ void __launch_bounds__(kBwdThreads) k_sparsity(RegArgs a, const __gri
             accumulate_sample<DT>(b, q, g, f2);
             const float sigma = expf(f2[0].x);
             const float alpha = -expm1f(-sigma * b.delta);
-            const float scale = a.weight / (float)a.n;
+            const float scale = a.weight / (float)a.n_rays;
             term = scale * alpha;
             if (a.grad_grid) {
                 float *const gp[3] = {a.grad_planes[3 * id], a.grad_planes[3 * id + 1], a.grad_planes[3 * id + 2]};
@@ -501,63 +584,91 @@ __global__ void __launch_bounds__(kBwdThreads) k_sparsity(RegArgs a, const __gri
             }
         }
     }
-    add_loss(term, a.loss);
+    term = cta_sum(term);
+    if (threadIdx.x == 0 && a.loss) atomicAdd(a.loss, term);
 }
 
+// Opacity, one ray per warp.  Bound by the L2's scattered reductions (65537 BF16
+// rays: a step of 8.4 ms, 12.1 ms with one ray per thread and 20 reductions a
+// sample).
 template <int DT>
-__global__ void __launch_bounds__(kBwdThreads, COW_REG_MIN_BLOCKS) k_opacity(RegArgs a,
+__global__ void __launch_bounds__(kBwdThreads, COW_REG_MIN_BLOCKS) k_opacity(const __grid_constant__ RegArgs a,
                                                                           const __grid_constant__ RayRecs rr) {
-    const int64_t t = (int64_t)blockIdx.x * kBwdThreads + threadIdx.x;
+    __shared__ BwdScratch s_bs[kBwdWarps];
+    BwdScratch &bs = s_bs[threadIdx.x >> 5];
+    WarpScratch &ws = bs.w;
+    const int lane = threadIdx.x & 31;
     float term = 0.f;
-    if (t < a.n) {
-        const int64_t r = a.ray_perm ? (int64_t)__ldg(a.ray_perm + t) : t;
-        float o[3], d[3];
-#pragma unroll
-        for (int c = 0; c < 3; c++) {
-            o[c] = __ldg(a.ray_o + 3 * r + c);
-            d[c] = __ldg(a.ray_d + 3 * r + c);
-        }
-        int order[kMaxRayIds];
-        const int n = sort_blocks_for_ray(rr, o, order);
-        float inv_d[3], omax;
+    const float scale = a.weight / (float)a.n_rays, eps = 1e-6f;
+    for (int64_t ray = first_ray(); ray < a.n_rays; ray += (int64_t)gridDim.x * kBwdWarps) {
+        float o[3], d[3], inv_d[3], omax;
+        const int64_t r = load_ray_warp(a, ray, o, d);
         ray_setup(d, o, inv_d, omax);
-        const float scale = a.weight / (float)a.n, eps = 1e-6f;
-        for (int k = 0; k < n; k++) {
-            const int id = rr.id[order[k]];
-            const BlockRec &b = rr.r[order[k]];
+        __syncwarp();
+        const int n = sort_blocks_warp(ws, rr, o);
+        for_each_hit(n, [&](int k) -> const BlockRec & { return rr.r[ws.ord[k]]; }, o, d, inv_d, [&](int k) {
+            const int pos = ws.ord[k], id = rr.id[pos];
+            const BlockRec &b = rr.r[pos];
             float T = 1.f;
             if (a.block_T) {  // the forward's in-block transmittance
-                T = __ldg(a.block_T + r * rr.n + order[k]);
-                if (T < 0.f) continue;  // no occupied sample
+                T = __ldg(a.block_T + r * rr.n + pos);
+                if (T < 0.f) return true;  // no occupied sample
             } else {
                 int nk = 0;
                 BrickCache bc;
-                for_each_sample(b, o, d, inv_d, omax, a.err, [&](const float p[3], const float g[3], float delta) {
-                    float2 f2[4];
-                    accumulate_sample<DT>(b, p, g, f2, &bc);
-                    T *= expf(-expf(f2[0].x) * delta);
-                    nk++;
+                for_each_chunk(ws, b, o, d, inv_d, omax, a.err,
+                               [&](bool active, int m, const float p[3], const float g[3], float delta) {
+                    float e = 1.f;
+                    if (active) {
+                        float2 f2[4];
+                        accumulate_sample<DT>(b, p, g, f2, &bc);
+                        e = expf(-expf(f2[0].x) * delta);
+                    }
+                    ws.row[7][lane] = e;
+                    __syncwarp();
+                    const float4 *e4 = reinterpret_cast<const float4 *>(ws.row[7]);
+                    for (int q = 0; 4 * q < m; q++) {
+                        const float4 e = e4[q];
+                        T = (((T * e.x) * e.y) * e.z) * e.w;
+                    }
+                    __syncwarp();
+                    nk += m;
                     return true;
                 });
-                if (nk == 0) continue;
+                if (nk == 0) return true;
             }
             const float a_raw = 1.f - T;
             const float al = fminf(fmaxf(a_raw, eps), 1.f - eps);
             term -= scale * (al * logf(al) + (1.f - al) * log1pf(-al));
-            if (!a.grad_grid || !(a_raw > eps && a_raw < 1.f - eps)) continue;
+            if (!a.grad_grid || !(a_raw > eps && a_raw < 1.f - eps)) return true;
             const float ga = -scale * (logf(al) - log1pf(-al));  // d loss / d alpha^k
-            float *gg = a.grad_grid[id];
             float *const gp[3] = {a.grad_planes[3 * id], a.grad_planes[3 * id + 1], a.grad_planes[3 * id + 2]};
             BrickCache bc;
-            for_each_sample(b, o, d, inv_d, omax, a.err, [&](const float p[3], const float g[3], float delta) {
-                float2 f2[4];
-                accumulate_sample<DT>(b, p, g, f2, &bc);
-                scatter_ch0(b, gg, gp, p, g, ga * expf(f2[0].x) * delta * T);
+            for_each_chunk(ws, b, o, d, inv_d, omax, a.err,
+                           [&](bool active, int m, const float p[3], const float g[3], float delta) {
+                float g0 = 0.f;
+                if (active) {
+                    float2 f2[4];
+                    accumulate_sample<DT>(b, p, g, f2, &bc);
+                    g0 = ga * expf(f2[0].x) * delta * T;
+                }
+                scatter_density_chunk(b, bs.tap, m, p, g, g0, a.grad_grid[id], gp);
                 return true;
             });
-        }
+            return true;
+        });
     }
-    add_loss(term, a.loss);
+    term = cta_sum(lane == 0 ? term : 0.f);
+    if (threadIdx.x == 0) a.loss_parts[blockIdx.x] = term;
+}
+
+// *loss += the CTAs' sums (in a fixed order: thousands of additions to one
+// float would cost its last bits)
+__global__ void __launch_bounds__(1024) k_add_parts(const float *__restrict__ parts, int n, float *loss) {
+    float v = 0.f;
+    for (int k = threadIdx.x; k < n; k += 1024) v += parts[k];
+    v = cta_sum(v);
+    if (threadIdx.x == 0) atomicAdd(loss, v);
 }
 
 // grad_mlp[t] += sum over CTA rows, in row order
@@ -633,7 +744,7 @@ __global__ void __launch_bounds__(kBwdThreads) k_bm_pass1(const __grid_constant_
     WarpScratch &ws = s_ws[threadIdx.x >> 5];
     const int lane = threadIdx.x & 31;
     float o[3], d[3], inv_d[3], omax;
-    const int64_t r = load_ray_warp(a, o, d);
+    const int64_t r = load_ray_warp(a, first_ray(), o, d);
     if (r < 0) return;
     ray_setup(d, o, inv_d, omax);
     const int n = sort_blocks_warp(ws, rr, o);
@@ -808,7 +919,7 @@ __global__ void __launch_bounds__(kBwdThreads, COW_BWD_MIN_BLOCKS) k_bm_remarch(
     BwdScratch &bs = s_bs[threadIdx.x >> 5];
     const int lane = threadIdx.x & 31;
     float o[3], d[3], inv_d[3], omax;
-    const int64_t r = load_ray_warp(a, o, d);
+    const int64_t r = load_ray_warp(a, first_ray(), o, d);
     if (r < 0) return;
     ray_setup(d, o, inv_d, omax);
     const float *S = a.S + 8 * r * a.n_ids, *G = a.G + 8 * r * a.n_ids;
@@ -884,8 +995,8 @@ cudaError_t launch_backward_block_mlps(const BmBwdArgs &a, const RayRecs &rr, cu
 }
 
 cudaError_t launch_sparsity(const RegArgs &a, const RayRecs &rr, cudaStream_t st) {
-    if (a.n <= 0) return cudaSuccess;
-    const int nb = (int)((a.n + kBwdThreads - 1) / kBwdThreads);
+    if (a.n_rays <= 0) return cudaSuccess;
+    const int nb = (int)((a.n_rays + kBwdThreads - 1) / kBwdThreads);
     {
         const cudaError_t e_ = dispatch_dt(a.dtype, [&](auto D) {
             k_sparsity<decltype(D)::value><<<nb, kBwdThreads, 0, st>>>(a, rr);
@@ -897,15 +1008,17 @@ cudaError_t launch_sparsity(const RegArgs &a, const RayRecs &rr, cudaStream_t st
 }
 
 cudaError_t launch_opacity(const RegArgs &a, const RayRecs &rr, cudaStream_t st) {
-    if (a.n <= 0) return cudaSuccess;
-    const int nb = (int)((a.n + kBwdThreads - 1) / kBwdThreads);
+    if (a.n_rays <= 0) return cudaSuccess;
+    // one ray per warp; beyond kOpacityMaxCtas CTAs (8 waves) one ray after another
+    const unsigned nw = (unsigned)std::min<int64_t>((a.n_rays + kBwdWarps - 1) / kBwdWarps, kOpacityMaxCtas);
     {
         const cudaError_t e_ = dispatch_dt(a.dtype, [&](auto D) {
-            k_opacity<decltype(D)::value><<<nb, kBwdThreads, 0, st>>>(a, rr);
+            k_opacity<decltype(D)::value><<<nw, kBwdThreads, 0, st>>>(a, rr);
             return cudaSuccess;
         });
         if (e_ != cudaSuccess) return e_;
     }
+    if (a.loss) k_add_parts<<<1, 1024, 0, st>>>(a.loss_parts, (int)nw, a.loss);
     return cudaGetLastError();
 }
 

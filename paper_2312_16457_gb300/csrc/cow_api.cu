@@ -826,7 +826,7 @@ cow_status cow_load_blocks_ex(cow_ctx **out, const cow_block_desc *blocks, int32
     if (any_host) e = cudaMalloc(&staging, max_vec * 32);
     if (e == cudaSuccess) e = cudaMalloc((void **)&d_amax, 8 * sizeof(unsigned));
     if (e == cudaSuccess) e = cudaMalloc((void **)&d_inv, 8 * sizeof(float));
-    if (e == cudaSuccess) e = cudaMalloc((void **)&c->d_err, sizeof(unsigned));
+    if (e == cudaSuccess) e = cudaMalloc((void **)&c->d_err, cowi::kCtxWords * sizeof(unsigned));
     if (e == cudaSuccess) e = cudaMalloc((void **)&c->d_mlp, 512 * sizeof(float));
     if (e == cudaSuccess) e = cudaMemsetAsync(c->d_err, 0, sizeof(unsigned), st);
     if (e != cudaSuccess)
@@ -1440,7 +1440,7 @@ cow_status cow_sparsity_loss(cow_ctx *ctx, const float *points, int64_t n_points
     cow_status rc = reg_prepare(ctx, ids, n_ids, loss, grad_grid, grad_planes, st, a);
     if (rc != COW_OK) return rc;
     a.pts = points;
-    a.n = n_points;
+    a.n_rays = n_points;
     a.weight = weight;
     cow::RayRecs rr;
     make_ray_recs(ctx, ids, n_ids, rr);
@@ -1464,9 +1464,10 @@ cow_status cow_opacity_loss(cow_ctx *ctx, const float *o, const float *d, int64_
     if (block_T && !is_device_ptr(block_T)) return fail(COW_ERR_INVALID_ARG, "block_T must be device memory");
     a.ray_o = o;
     a.ray_d = d;
-    a.n = n_rays;
+    a.n_rays = n_rays;
     a.weight = weight;
     a.block_T = block_T;
+    a.loss_parts = (float *)(ctx->d_err + kCtxLossParts);
     if ((rc = ray_order(ctx, o, d, n_rays, ids, n_ids, st, &a.ray_perm)) != COW_OK) return rc;
     cow::RayRecs rr;
     make_ray_recs(ctx, ids, n_ids, rr);

@@ -121,18 +121,20 @@ cudaError_t launch_backward_block_mlps(const BmBwdArgs &a, const RayRecs &rr, cu
 // block opacity (Eq. 8) over rays
 struct RegArgs {                  // the blocks that take part come by value (RayRecs)
     int32_t dtype;
-    const float *pts;             // sparsity: n x 3 points
-    const float *ray_o, *ray_d;   // opacity: n x 3 rays
-    int64_t n;
-    float weight;                 // the loss and its gradient are scaled by weight / n
-    const float *block_T;         // opacity: the forward's n x n_ids in-block transmittances (-1: no
+    const float *pts;             // sparsity: n_rays x 3 points
+    const float *ray_o, *ray_d;   // opacity: n_rays x 3 rays
+    int64_t n_rays;               // points or rays
+    float weight;                 // the loss and its gradient are scaled by weight / n_rays
+    const float *block_T;         // opacity: the forward's n_rays x n_ids in-block transmittances (-1: no
                                   // sample), or null to march every block twice
     float *loss;                  // device float, accumulated (may be null)
+    float *loss_parts;            // opacity: scratch, kOpacityMaxCtas floats
     float *const *grad_grid;      // device pointer table as in BwdArgs (null: no gradient)
     float *const *grad_planes;
     unsigned *err;
-    const int32_t *ray_perm;      // opacity, may be null: thread t takes ray ray_perm[t]
+    const int32_t *ray_perm;      // opacity, may be null: warp t takes ray ray_perm[t]
 };
+constexpr int kOpacityMaxCtas = 152 * 32;
 cudaError_t launch_sparsity(const RegArgs &a, const RayRecs &rr, cudaStream_t st);
 cudaError_t launch_opacity(const RegArgs &a, const RayRecs &rr, cudaStream_t st);
 // threads per CTA of the backward kernels: one MLP-gradient scratch row per

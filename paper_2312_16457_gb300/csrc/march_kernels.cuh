@@ -308,7 +308,7 @@ __global__ void __launch_bounds__(kThreads, COW_RAYS_MIN_BLOCKS) k_march_rays(co
     WarpScratch &ws = s_ws[threadIdx.x >> 5];
     const int lane = threadIdx.x & 31;
     float o[3], d[3], inv_d[3], omax;
-    const int64_t r = load_ray_warp(a, o, d);
+    const int64_t r = load_ray_warp(a, first_ray(), o, d);
     if (r < 0) return;
     ray_setup(d, o, inv_d, omax);
     // per-ray depth order: xy distance of block centres to this origin (App. D)
@@ -362,7 +362,7 @@ __global__ void __launch_bounds__(kThreads, COW_RAYS_MIN_BLOCKS) k_march_partial
     WarpScratch &ws = s_ws[threadIdx.x >> 5];
     const int lane = threadIdx.x & 31;
     float o[3], d[3], inv_d[3], omax;
-    const int64_t r = load_ray_warp(a, o, d);
+    const int64_t r = load_ray_warp(a, first_ray(), o, d);
     if (r < 0) return;
     ray_setup(d, o, inv_d, omax);
     float *pp = a.out_partials + 8 * r * rr.n;

@@ -290,11 +290,12 @@ __device__ __forceinline__ void for_each_hit(int n, RecAt rec_at, const float o[
     }
 }
 
-// The ray this warp marches, or -1 (a: the ray arrays and the order of a
-// ray-batch call).
+// Ray t in the call's order (a: the ray arrays and the order of a ray-batch
+// call): its index, or -1 beyond the last.
+__device__ __forceinline__ int64_t first_ray() { return (int64_t)blockIdx.x * (blockDim.x >> 5) + (threadIdx.x >> 5); }
+
 template <class Args>
-__device__ __forceinline__ int64_t load_ray_warp(const Args &a, float o[3], float d[3]) {
-    const int64_t t = (int64_t)blockIdx.x * (blockDim.x >> 5) + (threadIdx.x >> 5);
+__device__ __forceinline__ int64_t load_ray_warp(const Args &a, int64_t t, float o[3], float d[3]) {
     if (t >= a.n_rays) return -1;
     const int64_t r = a.ray_perm ? (int64_t)__ldg(a.ray_perm + t) : t;
 #pragma unroll

@@ -226,7 +226,7 @@ cow_status cow_load_scene(cow_ctx **out, const char *path, void *stream) {
     c->occ_thresh = h.occ_thresh;
     c->blocks.resize(table.size());
     cudaStream_t st = (cudaStream_t)stream;
-    cudaError_t e = cudaMalloc((void **)&c->d_err, sizeof(unsigned));
+    cudaError_t e = cudaMalloc((void **)&c->d_err, cowi::kCtxWords * sizeof(unsigned));
     if (e == cudaSuccess) e = cudaMalloc((void **)&c->d_mlp, 512 * sizeof(float));
     if (e == cudaSuccess) e = cudaMemset(c->d_err, 0, sizeof(unsigned));
     if (e != cudaSuccess) return bail(fail(COW_ERR_OOM, "cow_load_scene: %s", cudaGetErrorString(e)));
