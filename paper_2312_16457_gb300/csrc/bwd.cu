@@ -102,11 +102,11 @@ __device__ __forceinline__ void flush_half(float *dst, float2 acc[2]) {
     acc[0] = acc[1] = make_float2(0.f, 0.f);
 }
 
-// Put lane j's sample (j < n; point p, grid coordinate g, gradient gf) into
+// Put lane j's sample (j < n; lookup coordinates rel and g, gradient gf) into
 // tap[j]; ends: where the chunk's runs of samples in one voxel end, pends[k]:
 // in one texel cell of plane k.
 template <int NCH>
-__device__ __forceinline__ void make_taps(const BlockRec &b, TapRec *tap, int n, const float p[3], const float g[3],
+__device__ __forceinline__ void make_taps(const BlockRec &b, TapRec *tap, int n, const float rel[3], const float g[3],
                                           const float gf[NCH], unsigned &ends, unsigned pends[3]) {
     const int lane = threadIdx.x & 31;
     uint64_t base = 0;
@@ -116,11 +116,8 @@ __device__ __forceinline__ void make_taps(const BlockRec &b, TapRec *tap, int n,
         float fr[3], hf[3];
 #pragma unroll
         for (int a = 0; a < 3; a++) {
-            c0[a] = min(max(__float2int_rd(g[a]), 0), b.R - 2);
-            fr[a] = fminf(fmaxf(g[a], 0.f), (float)(b.R - 1)) - (float)c0[a];
-            const float h = axis_coord(p[a], b.plo[a], b.kp[a]);
-            h0[a] = min(max(__float2int_rd(h), 0), b.P - 2);
-            hf[a] = fminf(fmaxf(h, 0.f), (float)(b.P - 1)) - (float)h0[a];
+            c0[a] = lookup_cell(g[a], b.R, fr[a]);
+            h0[a] = lookup_cell(__fmul_rn(rel[a], b.kp[a]), b.P, hf[a]);
         }
         base = ((uint64_t)c0[2] * b.R + c0[1]) * b.R + c0[0];
         // below 2^32: a plane of more texels, with its gradient, exceeds the device
@@ -146,19 +143,19 @@ __device__ __forceinline__ void make_taps(const BlockRec &b, TapRec *tap, int n,
     __syncwarp();
 }
 
-// Scatter a chunk of n samples (lane j < n holds sample j's point and gradient
-// gf) to the taps of their lookups, as a warp: a lane has one tap and one half
+// Scatter a chunk of n samples (lane j < n holds sample j's lookup coordinates
+// and gradient gf) to the taps of their lookups, as a warp: a lane has one tap and one half
 // of its eight channels, so the lanes of one reduction cover whole 64-byte
 // vertex or texel pairs (the L2 takes 64-byte groups of float4 reductions 1.6
 // times as fast as scattered ones: 330 against 205 G/s into 32 MiB, 147 against
 // 46 G/s into 256 MiB), and it walks its samples in ray order, adding up what
 // goes to one voxel or texel cell before it issues the reduction (a lattice
 // step is about a quarter of a voxel, so a voxel takes some 2.5 samples).
-__device__ __forceinline__ void scatter_chunk(const BlockRec &b, TapRec *tap, int n, const float p[3],
+__device__ __forceinline__ void scatter_chunk(const BlockRec &b, TapRec *tap, int n, const float rel[3],
                                               const float g[3], const float gf[8], float *gg, float *const gp[3]) {
     const int lane = threadIdx.x & 31;
     unsigned ends, pends[3];
-    make_taps<8>(b, tap, n, p, g, gf, ends, pends);
+    make_taps<8>(b, tap, n, rel, g, gf, ends, pends);
     // place q (0 or 1) of an axis: weight 1 - f or f, as s f + c
     const float s1 = (lane & 2) ? 1.f : -1.f, c1 = (lane & 2) ? 0.f : 1.f;
     const float s2 = (lane & 4) ? 1.f : -1.f, c2 = (lane & 4) ? 0.f : 1.f;
@@ -210,11 +207,11 @@ __device__ __forceinline__ void scatter_chunk(const BlockRec &b, TapRec *tap, in
 
 // The same for the density channel alone: 8 lanes a run, one vertex each, then
 // one texel of the xy and xz planes each; 4 lanes a run for the yz plane.
-__device__ __forceinline__ void scatter_density_chunk(const BlockRec &b, TapRec *tap, int n, const float p[3],
+__device__ __forceinline__ void scatter_density_chunk(const BlockRec &b, TapRec *tap, int n, const float rel[3],
                                                       const float g[3], float g0, float *gg, float *const gp[3]) {
     const int lane = threadIdx.x & 31;
     unsigned ends, pends[3];
-    make_taps<1>(b, tap, n, p, g, &g0, ends, pends);
+    make_taps<1>(b, tap, n, rel, g, &g0, ends, pends);
     const bool a0 = lane & 1, a1 = lane & 2, a2 = lane & 4;
     const float s0 = a0 ? 1.f : -1.f, c0 = a0 ? 0.f : 1.f, s1 = a1 ? 1.f : -1.f, c1 = a1 ? 0.f : 1.f;
     const unsigned all = kFullMask >> (32 - n);
@@ -297,12 +294,12 @@ __device__ __forceinline__ bool remarch_block(BwdScratch &bs, const BlockRec &b,
     const int lane = threadIdx.x & 31;
     WarpScratch &ws = bs.w;
     BrickCache bc;
-    return for_each_chunk(ws, b, o, d, inv_d, omax, err, [&](bool active, int n, const float p[3], const float g[3],
+    return for_each_chunk(ws, b, o, d, inv_d, omax, err, [&](bool active, int n, const float rel[3], const float g[3],
                                                              float delta) {
         float e = 1.f, sigma = 0.f, gdot = 0.f, c[7] = {0.f, 0.f, 0.f, 0.f, 0.f, 0.f, 0.f};
         if (active) {
             float2 f2[4];
-            accumulate_sample<DT>(b, p, g, f2, &bc);
+            accumulate_sample<DT>(b, rel, g, f2, &bc);
             const float f[8] = {f2[0].x, f2[0].y, f2[1].x, f2[1].y, f2[2].x, f2[2].y, f2[3].x, f2[3].y};
             sigma = __expf(f[0]);
             e = __expf(-sigma * delta);
@@ -361,7 +358,7 @@ __device__ __forceinline__ bool remarch_block(BwdScratch &bs, const BlockRec &b,
 #pragma unroll
             for (int q = 0; q < 7; q++) gf[1 + q] = wt * gcf[q] * c[q] * (1.f - c[q]);
         }
-        scatter_chunk(b, bs.tap, used, p, g, gf, gg, gp);
+        scatter_chunk(b, bs.tap, used, rel, g, gf, gg, gp);
         return more;
     });
 }
@@ -496,17 +493,13 @@ __global__ void __launch_bounds__(kBwdThreads, COW_BWD_MIN_BLOCKS) k_remarch_bac
 // sample (8 grid vertices, 4 texels of each plane), in the opacity term added
 // up per voxel and texel cell first.
 
-__device__ __forceinline__ void scatter_ch0(const BlockRec &b, float *gg, float *const gp[3], const float p[3],
+__device__ __forceinline__ void scatter_ch0(const BlockRec &b, float *gg, float *const gp[3], const float rel[3],
                                             const float g[3], float g0) {
     if (gg) {
         float fr[3];
         int c0[3];
 #pragma unroll
-        for (int a = 0; a < 3; a++) {
-            const int v = min(max(__float2int_rd(g[a]), 0), b.R - 2);
-            c0[a] = v;
-            fr[a] = fminf(fmaxf(g[a], 0.f), (float)(b.R - 1)) - (float)v;
-        }
+        for (int a = 0; a < 3; a++) c0[a] = lookup_cell(g[a], b.R, fr[a]);
         const int64_t R = b.R;
         const int64_t base = (c0[2] * R + c0[1]) * R + c0[0];
 #pragma unroll
@@ -519,13 +512,7 @@ __device__ __forceinline__ void scatter_ch0(const BlockRec &b, float *gg, float 
     float hf[3];
     int h0[3];
 #pragma unroll
-    for (int a = 0; a < 3; a++) {
-        float h = axis_coord(p[a], b.plo[a], b.kp[a]);
-        const int u = min(max(__float2int_rd(h), 0), b.P - 2);
-        h = fminf(fmaxf(h, 0.f), (float)(b.P - 1));
-        h0[a] = u;
-        hf[a] = h - (float)u;
-    }
+    for (int a = 0; a < 3; a++) h0[a] = lookup_cell(__fmul_rn(rel[a], b.kp[a]), b.P, hf[a]);
     const int64_t P = b.P;
 #pragma unroll
     for (int pl = 0; pl < 3; pl++) {
@@ -617,11 +604,11 @@ __global__ void __launch_bounds__(kBwdThreads, COW_REG_MIN_BLOCKS) k_opacity(con
                 int nk = 0;
                 BrickCache bc;
                 for_each_chunk(ws, b, o, d, inv_d, omax, a.err,
-                               [&](bool active, int m, const float p[3], const float g[3], float delta) {
+                               [&](bool active, int m, const float rel[3], const float g[3], float delta) {
                     float e = 1.f;
                     if (active) {
                         float2 f2[4];
-                        accumulate_sample<DT>(b, p, g, f2, &bc);
+                        accumulate_sample<DT>(b, rel, g, f2, &bc);
                         e = expf(-expf(f2[0].x) * delta);
                     }
                     ws.row[7][lane] = e;
@@ -645,14 +632,14 @@ __global__ void __launch_bounds__(kBwdThreads, COW_REG_MIN_BLOCKS) k_opacity(con
             float *const gp[3] = {a.grad_planes[3 * id], a.grad_planes[3 * id + 1], a.grad_planes[3 * id + 2]};
             BrickCache bc;
             for_each_chunk(ws, b, o, d, inv_d, omax, a.err,
-                           [&](bool active, int m, const float p[3], const float g[3], float delta) {
+                           [&](bool active, int m, const float rel[3], const float g[3], float delta) {
                 float g0 = 0.f;
                 if (active) {
                     float2 f2[4];
-                    accumulate_sample<DT>(b, p, g, f2, &bc);
+                    accumulate_sample<DT>(b, rel, g, f2, &bc);
                     g0 = ga * expf(f2[0].x) * delta * T;
                 }
-                scatter_density_chunk(b, bs.tap, m, p, g, g0, a.grad_grid[id], gp);
+                scatter_density_chunk(b, bs.tap, m, rel, g, g0, a.grad_grid[id], gp);
                 return true;
             });
             return true;

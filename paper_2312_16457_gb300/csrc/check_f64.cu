@@ -82,7 +82,7 @@ __global__ void __launch_bounds__(kF64Threads) k_march_rays_f64(F64Args a, const
         const int id = rr.id[order[k]];
         const double *grid = a.grids[id];
         const double *const planes[3] = {a.planes[3 * id], a.planes[3 * id + 1], a.planes[3 * id + 2]};
-        for_each_sample(b, o, d, inv_d, omax, a.err, [&](const float q[3], const float *, float step) {
+        for_each_sample(b, o, d, inv_d, omax, a.err, [&](const float q[3], const float *, const float *, float step) {
             double f[8];
             feature64(b, grid, planes, q, f);
             const double sigma = exp(f[0]);

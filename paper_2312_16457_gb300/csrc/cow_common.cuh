@@ -182,9 +182,6 @@ __device__ __forceinline__ bool inside_block(const BlockRec &b, const float p[3]
            p[2] <= b.hi[2];
 }
 
-// Continuous vertex coordinate along one axis: (p - lo) * k.
-__device__ __forceinline__ float axis_coord(float p, float lo, float k) { return __fmul_rn(__fsub_rn(p, lo), k); }
-
 // --- unbounded blocks: the region they own and the contraction (Eq. 16) -----
 // The block owns its xy footprint extended to infinity across the sides in
 // b.unb (half-open as Eq. 4) and every z.
@@ -221,19 +218,42 @@ __device__ __forceinline__ void contract_u(const float x[3], float m, float u[3]
     }
 }
 
-// Lookup coordinates of a point for the feature gathers: q (the point, or
-// its contraction u for an unbounded block) and the grid coordinate g.
-__device__ __forceinline__ void lookup_coords(const BlockRec &b, const float p[3], float q[3], float g[3]) {
-    if (b.unb & kUnbContracted) {
-        float x[3];
-        const float m = unbounded_x(b, p, x);
-        contract_u(x, m, q);
-    } else {
+// Lookup coordinates of a point the block owns: rel, its offset from the
+// origin of the lookup (lo; -2 for the contraction u of an unbounded block),
+// and the grid coordinate g.  Both are >= 0; a NaN coordinate of an unbounded
+// block's point looks up at 0.
+__device__ __forceinline__ void lookup_u(const BlockRec &b, const float u[3], float rel[3], float g[3]) {
 #pragma unroll
-        for (int a = 0; a < 3; a++) q[a] = p[a];
+    for (int a = 0; a < 3; a++) {
+        rel[a] = fmaxf(__fsub_rn(u[a], b.plo[a]), 0.f);
+        g[a] = __fmul_rn(rel[a], b.kg[a]);
     }
+}
+
+__device__ __forceinline__ void lookup_p(const BlockRec &b, const float p[3], float rel[3], float g[3]) {
 #pragma unroll
-    for (int a = 0; a < 3; a++) g[a] = axis_coord(q[a], b.plo[a], b.kg[a]);
+    for (int a = 0; a < 3; a++) {
+        rel[a] = __fsub_rn(p[a], b.lo[a]);
+        g[a] = __fmul_rn(rel[a], b.kg[a]);
+    }
+}
+
+__device__ __forceinline__ void lookup_coords(const BlockRec &b, const float p[3], float rel[3], float g[3]) {
+    if (b.unb & kUnbContracted) {
+        float x[3], u[3];
+        const float m = unbounded_x(b, p, x);
+        contract_u(x, m, u);
+        lookup_u(b, u, rel, g);
+    } else {
+        lookup_p(b, p, rel, g);
+    }
+}
+
+// Vertex below a lookup coordinate x >= 0 (n vertices) and the place behind it.
+__device__ __forceinline__ int lookup_cell(float x, int n, float &frac) {
+    const int v = min(__float2int_rd(x), n - 2);
+    frac = fminf(x, (float)(n - 1)) - (float)v;
+    return v;
 }
 
 // Candidate lattice range of a ray in a block: FP32 slab test on the grown

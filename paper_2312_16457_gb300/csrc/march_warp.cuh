@@ -27,7 +27,7 @@ struct alignas(16) WarpScratch {
 };
 
 // Occupied lattice samples of the warp's ray inside block b, in order, 32 at a
-// time: fn(active, n, p, g, s) is called with lanes 0 .. n-1 holding one sample
+// time: fn(active, n, rel, g, s) is called with lanes 0 .. n-1 holding one sample
 // each (n = 32 except for the block's last call); it returns false (uniformly)
 // to stop the ray.  The lattice is scanned 32 points at a step, occupied points
 // are queued, and a chunk is handed out when 32 are there, so empty space costs
@@ -82,14 +82,15 @@ __device__ __forceinline__ bool for_each_chunk(WarpScratch &ws, const BlockRec &
                     t_next = __fadd_rn(t_next, __fmul_rn(__fmul_rn(delta, m1), m1));
                 }
                 if (lane < k) {
-                    float p[3], x[3], u[3];
+                    float p[3], x[3], u[3], rel[3], g[3];
 #pragma unroll
                     for (int a = 0; a < 3; a++) p[a] = __fadd_rn(o[a], __fmul_rn(tl, d[a]));
                     contract_u(x, unbounded_x(b, p, x), u);
+                    lookup_u(b, u, rel, g);
                     int cell[3];
 #pragma unroll
                     for (int a = 0; a < 3; a++) {
-                        const int v = min(max(__float2int_rd(axis_coord(u[a], b.plo[a], b.kg[a])), 0), R - 2);
+                        const int v = min(__float2int_rd(g[a]), R - 2);
                         cell[a] = C == 1 ? v : (int)__umulhi((unsigned)v, b.cdiv);
                     }
                     const int ci = (cell[2] * Nc + cell[1]) * Nc + cell[0];
@@ -103,10 +104,12 @@ __device__ __forceinline__ bool for_each_chunk(WarpScratch &ws, const BlockRec &
                     float p[3];
                     lattice_point(o, d, delta, item, p);
                     if (inside_block(b, p)) {
+                        float rel[3], g[3];
+                        lookup_p(b, p, rel, g);
                         int cell[3];
 #pragma unroll
                         for (int a = 0; a < 3; a++) {
-                            const int v = min(max(__float2int_rd(axis_coord(p[a], b.lo[a], b.kg[a])), 0), R - 2);
+                            const int v = min(__float2int_rd(g[a]), R - 2);
                             cell[a] = C == 1 ? v : (int)__umulhi((unsigned)v, b.cdiv);
                         }
                         const int ci = (cell[2] * Nc + cell[1]) * Nc + cell[0];
@@ -132,7 +135,7 @@ __device__ __forceinline__ bool for_each_chunk(WarpScratch &ws, const BlockRec &
         __syncwarp();
         if (32 + lane < qn) ws.q[lane] = rest;
         qn -= n;
-        float p[3], g[3], s = delta;
+        float p[3], rel[3], g[3], s = delta;
         if (unb) {
             const float t = __int_as_float(item);
             float q[3], x[3];
@@ -141,14 +144,12 @@ __device__ __forceinline__ bool for_each_chunk(WarpScratch &ws, const BlockRec &
             const float mm = unbounded_x(b, q, x), m1 = fmaxf(mm, 1.f);
             s = __fmul_rn(__fmul_rn(delta, m1), m1);
             contract_u(x, mm, p);
-#pragma unroll
-            for (int a = 0; a < 3; a++) g[a] = axis_coord(p[a], b.plo[a], b.kg[a]);
+            lookup_u(b, p, rel, g);
         } else {
             lattice_point(o, d, delta, item, p);
-#pragma unroll
-            for (int a = 0; a < 3; a++) g[a] = axis_coord(p[a], b.lo[a], b.kg[a]);
+            lookup_p(b, p, rel, g);
         }
-        if (!fn(active, n, p, g, s)) return false;
+        if (!fn(active, n, rel, g, s)) return false;
     } while (qn > 0 || base <= last);
     return true;
 }
@@ -227,11 +228,11 @@ __device__ __forceinline__ void march_block_warp(WarpScratch &ws, const BlockRec
                                                  WarpRay &s, unsigned *err, float *tb = nullptr) {
     BrickCache bc;
     const bool more = for_each_chunk(ws, b, o, d, inv_d, omax, err,
-                                     [&](bool active, int n, const float p[3], const float g[3], float dt) {
+                                     [&](bool active, int n, const float rel[3], const float g[3], float dt) {
         float e = 1.f, c[7] = {0.f, 0.f, 0.f, 0.f, 0.f, 0.f, 0.f};
         if (active) {
             float2 f2[4];
-            accumulate_sample<DT>(b, p, g, f2, &bc);
+            accumulate_sample<DT>(b, rel, g, f2, &bc);
             const float f[8] = {f2[0].x, f2[0].y, f2[1].x, f2[1].y, f2[2].x, f2[2].y, f2[3].x, f2[3].y};
             e = __expf(-__expf(f[0]) * dt);
 #pragma unroll
