@@ -602,26 +602,19 @@ __global__ void __launch_bounds__(kBwdThreads, COW_REG_MIN_BLOCKS) k_opacity(con
                 if (T < 0.f) return true;  // no occupied sample
             } else {
                 int nk = 0;
+                float tau = 0.f;  // this lane's samples (march_block_warp)
                 BrickCache bc;
                 for_each_chunk(ws, b, o, d, inv_d, omax, a.err,
                                [&](bool active, int m, const float rel[3], const float g[3], float delta) {
-                    float e = 1.f;
                     if (active) {
                         float2 f2[4];
                         accumulate_sample<DT>(b, rel, g, f2, &bc);
-                        e = expf(-expf(f2[0].x) * delta);
+                        tau += expf(f2[0].x) * delta;
                     }
-                    ws.row[7][lane] = e;
-                    __syncwarp();
-                    const float4 *e4 = reinterpret_cast<const float4 *>(ws.row[7]);
-                    for (int q = 0; 4 * q < m; q++) {
-                        const float4 e = e4[q];
-                        T = (((T * e.x) * e.y) * e.z) * e.w;
-                    }
-                    __syncwarp();
                     nk += m;
                     return true;
                 });
+                T = expf(-warp_sum(tau));
                 if (nk == 0) return true;
             }
             const float a_raw = 1.f - T;

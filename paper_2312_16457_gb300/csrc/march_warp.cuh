@@ -19,6 +19,12 @@ namespace cow {
 constexpr unsigned kFullMask = 0xffffffffu;
 constexpr int kRowPad = 36;  // row stride: the float4 reads of 8 rows fall into distinct banks
 
+__device__ __forceinline__ float warp_sum(float x) {
+#pragma unroll
+    for (int off = 16; off > 0; off >>= 1) x += __shfl_xor_sync(kFullMask, x, off);
+    return x;
+}
+
 // Shared scratch of one warp.
 struct alignas(16) WarpScratch {
     float row[8][kRowPad];   // channels 0-6 of the chunk's samples, then exp(-sigma delta)
@@ -174,10 +180,9 @@ __device__ __forceinline__ void chunk_weights(const float4 &e, float &T, float w
 
 // Composite a chunk of n samples (Eq. 1-2) in order: each lane brings its
 // sample's e = exp(-sigma s) and seven colours (e = 1, colours 0 beyond n,
-// which leave T and the sums as they are).  tb, when given, is multiplied by
-// every e.  Returns false once T < ert_eps, with the samples after it unused.
+// which leave T and the sums as they are).  Returns false once T < ert_eps, with the samples after it unused.
 __device__ __forceinline__ bool composite_chunk(WarpScratch &ws, int n, float e, const float c[7], float ert_eps,
-                                                WarpRay &s, float *tb = nullptr) {
+                                                WarpRay &s) {
     const int lane = threadIdx.x & 31;
 #pragma unroll
     for (int q = 0; q < 7; q++) ws.row[q][lane] = c[q];
@@ -185,7 +190,7 @@ __device__ __forceinline__ bool composite_chunk(WarpScratch &ws, int n, float e,
     __syncwarp();
     const float4 *x4 = reinterpret_cast<const float4 *>(ws.row[lane & 7]);
     const float4 *e4 = reinterpret_cast<const float4 *>(ws.row[7]);
-    float T = s.T, acc = s.acc, t = tb ? *tb : 0.f;
+    float T = s.T, acc = s.acc;
 #pragma unroll
     for (int k = 0; k < 8; k++) {
         if (4 * k >= n) break;
@@ -193,7 +198,6 @@ __device__ __forceinline__ bool composite_chunk(WarpScratch &ws, int n, float e,
         float w[4];
         chunk_weights(ee, T, w);
         acc = fmaf(w[3], xx.w, fmaf(w[2], xx.z, fmaf(w[1], xx.y, fmaf(w[0], xx.x, acc))));
-        if (tb) t = (((t * ee.x) * ee.y) * ee.z) * ee.w;
     }
     bool more = true;
     int used = n;
@@ -201,13 +205,11 @@ __device__ __forceinline__ bool composite_chunk(WarpScratch &ws, int n, float e,
         more = false;
         T = s.T;
         acc = s.acc;
-        t = tb ? *tb : 0.f;
         const float *er = ws.row[7], *xr = ws.row[lane & 7];
         for (used = 0; used < n;) {
             const float ev = er[used];
             acc = fmaf(T * (1.f - ev), xr[used], acc);
             T *= ev;
-            if (tb) t *= ev;
             used++;
             if (T < ert_eps) break;
         }
@@ -216,17 +218,20 @@ __device__ __forceinline__ bool composite_chunk(WarpScratch &ws, int n, float e,
     s.acc = acc;
     s.T = T;
     s.nsamp += used;
-    if (tb) *tb = t;
     return more;
 }
 
 // March the warp's ray through one block, updating its composite (march_block
-// of the one-ray-per-thread form).
+// of the one-ray-per-thread form).  tb, when given, receives the block's own
+// transmittance (Eq. 11) as exp(-sum of sigma s): the product of the rounded
+// 1 - alpha loses what thin samples take (the opacity term of 65537 rays: 5e-6
+// off in the product's form).
 template <int DT>
 __device__ __forceinline__ void march_block_warp(WarpScratch &ws, const BlockRec &b, const float o[3],
                                                  const float d[3], const float inv_d[3], float omax, float ert_eps,
                                                  WarpRay &s, unsigned *err, float *tb = nullptr) {
     BrickCache bc;
+    float tau = 0.f;  // this lane's samples
     const bool more = for_each_chunk(ws, b, o, d, inv_d, omax, err,
                                      [&](bool active, int n, const float rel[3], const float g[3], float dt) {
         float e = 1.f, c[7] = {0.f, 0.f, 0.f, 0.f, 0.f, 0.f, 0.f};
@@ -234,13 +239,16 @@ __device__ __forceinline__ void march_block_warp(WarpScratch &ws, const BlockRec
             float2 f2[4];
             accumulate_sample<DT>(b, rel, g, f2, &bc);
             const float f[8] = {f2[0].x, f2[0].y, f2[1].x, f2[1].y, f2[2].x, f2[2].y, f2[3].x, f2[3].y};
-            e = __expf(-__expf(f[0]) * dt);
+            const float sd = __expf(f[0]) * dt;
+            e = __expf(-sd);
+            tau += sd;
 #pragma unroll
             for (int q = 0; q < 7; q++) c[q] = sigmoidf_fast(f[1 + q]);
         }
-        return composite_chunk(ws, n, e, c, ert_eps, s, tb);
+        return composite_chunk(ws, n, e, c, ert_eps, s);
     });
     if (!more) s.done = true;
+    if (tb) *tb = expf(-warp_sum(tau));
 }
 
 // The call's blocks in the order of sort_blocks_for_ray (FP32 key, ties by id,
