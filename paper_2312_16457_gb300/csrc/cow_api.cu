@@ -261,6 +261,17 @@ cow_status pack_tensor(cow_ctx *c, BlockHost &b, int t, const float *s, const fl
 cow_status repack_block(cow_ctx *c, BlockHost &b, const float *const src_in[4], void *staging, unsigned *d_amax,
                         float *d_inv, cudaStream_t st) {
     const int64_t nv[4] = {(int64_t)b.R * b.R * b.R, (int64_t)b.P * b.P, (int64_t)b.P * b.P, (int64_t)b.P * b.P};
+    // dense FP32 / FP16 / BF16 from device masters: the scales are 1 and stay
+    // so, one launch packs the block
+    if (!c->bricks && (c->dtype == cow::kF32 || c->dtype == cow::kF16 || c->dtype == cow::kBF16) &&
+        is_device_ptr(src_in[0]) && is_device_ptr(src_in[1]) && is_device_ptr(src_in[2]) && is_device_ptr(src_in[3])) {
+        const cow::PackBlock a = {{src_in[0], src_in[1], src_in[2], src_in[3]},
+                                  {b.grid, b.planes[0], b.planes[1], b.planes[2]},
+                                  {nv[0], nv[1]},
+                                  {b.R, b.P}};
+        COW_CUDA(cow::launch_pack_block(a, c->dtype, st));
+        return COW_OK;
+    }
     float scale_h[32];
     for (int t = 0; t < 4; t++) {
         const float *s = src_in[t];

@@ -193,6 +193,14 @@ cudaError_t launch_amax8(const float *x, int64_t n_vec, unsigned *amax_bits, cud
 // (element i = vertex i and vertex i+1 of its row of `row` vertices).
 cudaError_t launch_pack(const float *x, int64_t n_vec, int row, int dtype, const float *inv_scale8, void *out,
                         cudaStream_t st);
+// The grid and planes of a dense block, FP32 / FP16 / BF16, in one launch.
+struct PackBlock {
+    const float *src[4];  // FP32 masters: grid, planes (16-byte aligned)
+    void *dst[4];
+    int64_t n[2];         // vertices of the grid, texels of one plane
+    int32_t row[2];       // R, P
+};
+cudaError_t launch_pack_block(const PackBlock &a, int dtype, cudaStream_t st);
 cudaError_t launch_occupancy(const float *grid, int R, int C, double log_thresh, uint32_t *bits, cudaStream_t st);
 cudaError_t launch_pack_quad8(const float *x, int P, const float *inv_scale8, void *out, cudaStream_t st);
 // Grid element layouts (k_pack_grid): one FP32 vertex; a vertex pair along x

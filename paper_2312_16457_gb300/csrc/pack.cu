@@ -101,6 +101,42 @@ __global__ void k_pack(const float *__restrict__ x, int64_t n_vec, int row, cons
     }
 }
 
+// The four tensors of a dense block in one launch, scale 1 (FP32, FP16, BF16):
+// a training step re-packs every block, and at the sizes of a mini-batch step
+// the launches and the copies of constant scales cost more than the bytes.
+template <int DT>
+__global__ void __launch_bounds__(256) k_pack_block(const __grid_constant__ PackBlock a) {
+    const int64_t n0 = a.n[0], n1 = a.n[1], total = n0 + 3 * n1;
+    for (int64_t e = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; e < total; e += (int64_t)gridDim.x * blockDim.x) {
+        int t = 0;
+        int64_t i = e;
+        if (i >= n0) {
+            i -= n0;
+            t = 1;
+            while (i >= n1) i -= n1, t++;
+        }
+        const int row = a.row[t > 0];
+        const float4 *x = reinterpret_cast<const float4 *>(a.src[t]);
+        const float4 v0 = __ldg(x + 2 * i), v1 = __ldg(x + 2 * i + 1);
+        if (DT == kF32) {
+            float4 *o = reinterpret_cast<float4 *>(a.dst[t]) + 2 * i;
+            o[0] = v0;
+            o[1] = v1;
+            continue;
+        }
+        const int64_t j = (i % row) == row - 1 ? i : i + 1;
+        const float4 u0 = __ldg(x + 2 * j), u1 = __ldg(x + 2 * j + 1);
+        const float v[8] = {v0.x, v0.y, v0.z, v0.w, v1.x, v1.y, v1.z, v1.w};
+        const float u[8] = {u0.x, u0.y, u0.z, u0.w, u1.x, u1.y, u1.z, u1.w};
+        uint32_t w[8];
+        encode8<DT>(v, w);
+        encode8<DT>(u, w + 4);
+        uint4 *o = reinterpret_cast<uint4 *>(a.dst[t]) + 2 * i;
+        o[0] = make_uint4(w[0], w[1], w[2], w[3]);
+        o[1] = make_uint4(w[4], w[5], w[6], w[7]);
+    }
+}
+
 __global__ void k_occupancy(const float *__restrict__ grid, int R, int C, int Nc, double lt, uint32_t *bits) {
     const int64_t ncell = (int64_t)Nc * Nc * Nc;
     for (int64_t c = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; c < ncell; c += (int64_t)gridDim.x * blockDim.x) {
@@ -258,6 +294,17 @@ cudaError_t launch_pack(const float *x, int64_t n_vec, int row, int dtype, const
     case kF16: k_pack<kF16><<<g, 256, 0, st>>>(x, n_vec, row, inv_scale8, out); break;
     case kBF16: k_pack<kBF16><<<g, 256, 0, st>>>(x, n_vec, row, inv_scale8, out); break;
     case kFP8: k_pack<kFP8><<<g, 256, 0, st>>>(x, n_vec, row, inv_scale8, out); break;
+    default: return cudaErrorInvalidValue;
+    }
+    return cudaGetLastError();
+}
+
+cudaError_t launch_pack_block(const PackBlock &a, int dtype, cudaStream_t st) {
+    const int g = grid_for(a.n[0] + 3 * a.n[1], 256);
+    switch (dtype) {
+    case kF32: k_pack_block<kF32><<<g, 256, 0, st>>>(a); break;
+    case kF16: k_pack_block<kF16><<<g, 256, 0, st>>>(a); break;
+    case kBF16: k_pack_block<kBF16><<<g, 256, 0, st>>>(a); break;
     default: return cudaErrorInvalidValue;
     }
     return cudaGetLastError();

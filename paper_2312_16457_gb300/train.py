@@ -15,6 +15,13 @@ import torch
 from . import cow
 
 
+def _zeros(shapes, device) -> List[torch.Tensor]:
+    """FP32 zeros of these shapes, filled by one multi-tensor launch."""
+    out = [torch.empty(s, dtype=torch.float32, device=device) for s in shapes]
+    torch._foreach_zero_(out)
+    return out
+
+
 class RenderRays(torch.autograd.Function):
     """rgb = render(o, d; features, mlp).  Inputs: the context, block ids, the
     MLP (499) and the flat feature parameters [grid_0, xy_0, xz_0, yz_0, grid_1,
@@ -37,7 +44,7 @@ class RenderRays(torch.autograd.Function):
         o, d, mlp, aux = fctx.saved_tensors
         cctx = fctx.cctx
         nb = cctx.n_blocks
-        grads = [torch.zeros(s, dtype=torch.float32, device=o.device) for s in fctx.shapes]
+        grads = _zeros(fctx.shapes, o.device)
         gm = torch.zeros(499, dtype=torch.float32, device=o.device)
         cctx.render_backward(o, d, fctx.ids, mlp.detach().contiguous(), aux, grad_rgb.contiguous().float(),
                              [grads[4 * i] for i in range(nb)], [grads[4 * i + 1:4 * i + 4] for i in range(nb)], gm,
@@ -110,7 +117,7 @@ class Fitter:
         else:
             rgb, aux, _ = self.ctx.render_rays(o, d, self.ids, self.mlp, ert_eps=ert_eps)
         g, loss = cow.mse_grad(rgb, target)
-        grads = [torch.zeros_like(p) for p in self.params]
+        grads = _zeros([p.shape for p in self.params], o.device)
         gtab = ([grads[4 * i] for i in range(nb)], [grads[4 * i + 1:4 * i + 4] for i in range(nb)])
         if per_block:
             gm = torch.zeros_like(self.block_mlps)
