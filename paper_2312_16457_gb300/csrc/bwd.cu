@@ -20,10 +20,10 @@
 //       natural layout).
 // K6's bound was the L2's rate of scattered reductions, 40 float4 a sample (one
 // ray per thread: 130 ms for 2^20 random rays over 2x2 blocks of 128^3 FP32,
-// 5.5e8 samples).  With a voxel's or texel's contributions added up before they
-// are reduced and the reductions in 64-byte groups it takes 73 ms; what bounds
-// it now is latency at 16 warps per SM (issue slots 37 % busy) with the L1 data
-// pipe 63 % and the L2 53 % busy, gathers and reductions together.
+// 5.6e8 samples).  With a voxel's or texel's contributions added up before they
+// are reduced and the reductions in 64-byte groups it takes 65 ms, of which 35
+// are the reductions (timed without them); the rest is latency at 20 warps per SM
+// (issue slots 37 % busy, L1 data pipe 63 %, L2 53 %).
 // The CTA's MLP weight gradient (499 sums over its 128 rays) goes to a
 // per-CTA scratch row; a second kernel adds the rows in a fixed order, so the
 // MLP gradient does not depend on scheduling.
@@ -40,8 +40,10 @@ namespace {
 
 #ifndef COW_BWD_MIN_BLOCKS
 // CTAs per SM the re-march's register budget is sized for: the 2^20-ray step
-// takes 142 ms at 2, 120 at 3, 107 at 4 and 106 at 5, which spills 80 bytes
-#define COW_BWD_MIN_BLOCKS 4
+// took 142 ms at 2, 120 at 3, 107 at 4; with the present ray order 97.0 at 4 and
+// 96.2 at 5, though that spills 16 to 40 bytes (100003 rays of the per-block MLP
+// form 10.8 and 10.6 ms, 65537 BF16 rays 8.85 and 8.66 ms); 6 was slower
+#define COW_BWD_MIN_BLOCKS 5
 #endif
 
 #ifndef COW_REG_MIN_BLOCKS
@@ -704,10 +706,11 @@ __global__ void __launch_bounds__(256) k_adam(float *__restrict__ p, const float
     for (int64_t i = 4 * n4 + t; i < n; i += step) adam_one(p[i], g[i], m[i], v[i], a);
 }
 
-__global__ void k_mse_grad(const float *__restrict__ rgb, const float *__restrict__ tgt, int64_t n, float scale,
+__global__ void __launch_bounds__(1024) k_mse_grad(const float *__restrict__ rgb, const float *__restrict__ tgt, int64_t n, float scale,
                            float *__restrict__ grad, float *loss) {
     __shared__ float s_part[32];
     float acc = 0.f;
+#pragma unroll 4
     for (int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; i < n; i += (int64_t)gridDim.x * blockDim.x) {
         const float e = rgb[i] - tgt[i];
         grad[i] = 2.f * scale * e;
@@ -1052,9 +1055,11 @@ cudaError_t launch_mse_grad(const float *rgb, const float *tgt, int64_t n, float
         cudaError_t e = cudaMemsetAsync(loss, 0, sizeof(float), st);
         if (e != cudaSuccess) return e;
     }
-    int64_t blocks = (n + 255) / 256;
-    if (blocks > 152 * 16) blocks = 152 * 16;
-    k_mse_grad<<<(int)blocks, 256, 0, st>>>(rgb, tgt, n, 1.0f / (float)n, grad, loss);
+    // one CTA of 32 warps per SM at most: every CTA adds its part to the loss, and
+    // the 2432 additions of 3.1 M values at 256 threads a CTA cost it 1.5e-6
+    int64_t blocks = (n + 1023) / 1024;
+    if (blocks > 152) blocks = 152;
+    k_mse_grad<<<(int)blocks, 1024, 0, st>>>(rgb, tgt, n, 1.0f / (float)n, grad, loss);
     return cudaGetLastError();
 }
 
