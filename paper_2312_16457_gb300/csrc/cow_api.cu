@@ -573,7 +573,13 @@ cow_status ray_order(cow_ctx *c, const float *o, const float *d, int64_t n, cons
     *perm = nullptr;
     if (alike) *alike = nullptr;
     const bool sort = c->ray_order == COW_RAY_ORDER_COHERENT && n >= kRayOrderMin;
-    const bool count = alike && n >= cow::kRaysAlikeMin;
+    bool count = alike && n >= cow::kRaysAlikeMin;
+    if (count && !sort && (c->ray_keys.cap < (size_t)n * sizeof(uint32_t) || !c->ray_hist.cap)) {
+        // the given order needs no scratch otherwise: none is allocated inside a capture
+        cudaStreamCaptureStatus cs = cudaStreamCaptureStatusNone;
+        if (cudaStreamIsCapturing(st, &cs) != cudaSuccess) cudaGetLastError();
+        if (cs != cudaStreamCaptureStatusNone) count = false;
+    }
     if (!(sort || count) || n > 0x7fffffff) return COW_OK;
     float lo[3] = {3.0e38f, 3.0e38f, 3.0e38f}, hi[3] = {-3.0e38f, -3.0e38f, -3.0e38f};
     for (int32_t k = 0; k < n_ids; k++) {
