@@ -38,17 +38,18 @@ METRIC = "1080p frames/s & Mrays/s: BF16/batched vs plain FP32 at >=45 dB PSNR"
 # with ncu (dram__bytes_read.sum + dram__bytes_write.sum) and keyed to the
 # SHA-256 of the sources that build the marcher: after any change to them the
 # stored number no longer describes the kernel and the line reports null.
-MARCH_SOURCES = ["march.cu", "march_kernels.cuh", "march_core.cuh", "cow_common.cuh", "cow_kernels.h", "kernel_launch.h"]
+MARCH_SOURCES = ["march.cu", "march_kernels.cuh", "march_core.cuh", "march_warp.cuh", "cow_common.cuh", "cow_kernels.h",
+                 "kernel_launch.h"]
 MEASURED_TRAFFIC = {  # (workload, storage, schedule, res_div) -> (bytes per launch, sources sha256)
     ("city_lod_1080p", "bf16", "thread_const", 1):
-        (49_420_000_000 + 25_720_000, "1b2344d4e053c5b72a13ade2ce1b515fdfa894f843b8547a0daecac5721b64c9"),
+        (49_834_812_416 + 25_886_208, "4f05223abd54a072c434688b4c9a3255192b7fdae0478e6780dc34c7a16e8a52"),
 }
 # The L1 data-pipe utilisation of the same kernel (ncu
 # l1tex__data_pipe_lsu_wavefronts.sum.pct_of_peak_sustained_elapsed, one
 # launch of the half-resolution bake of the workload), keyed the same way.
 MEASURED_L1_WAVEFRONTS = {  # (workload, storage, schedule) -> (fraction, sources sha256)
     ("city_lod_1080p", "bf16", "thread_const"):
-        (0.700, "1b2344d4e053c5b72a13ade2ce1b515fdfa894f843b8547a0daecac5721b64c9"),
+        (0.763, "4f05223abd54a072c434688b4c9a3255192b7fdae0478e6780dc34c7a16e8a52"),
 }
 # HBM copy bandwidth when the measured peaks file is absent: an earlier
 # measurement of a GB300's copy rate
@@ -683,8 +684,9 @@ def run_fit(args, ws, rank, local):
                "peak_gred_per_s_hbm": round(peak_red_hbm, 2),
                "peak_source": "measured live: random red.global.add.v4.f32 into a 32 MiB (L2-resident) buffer, "
                               "cow_reduce_peak",
-               "note": "time of the whole backward call (MLP backward + re-march); reductions counted as 40 per "
-                       "occupied sample"}
+               "note": "time of the whole backward call (MLP backward + re-march); reductions counted as the 40 "
+                       "float4 contributions of an occupied sample: the kernel adds up those of one voxel or "
+                       "texel cell and reduces in 64-byte groups, so the rate can exceed the probe's"}
     line = {"metric": "differentiation form: training rays/s (forward + backward + Adam)", "value": round(n / ms / 1e3, 3),
             "unit": "Mrays/s", "n_gpus": ws, "steps": args.steps, "warmup": args.warmup, "ms_per_step": round(ms, 3),
             "higher_is_better": True, "dtype": "f32", "data": "synthetic",
