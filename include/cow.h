@@ -666,10 +666,13 @@ cow_status cow_set_schedule(cow_ctx *ctx, int32_t schedule);
  * over 2x2 blocks of 128^3 / 512^2 FP32 features: forward 39.9 -> 28.3 ms).
  * COW_RAY_ORDER_GIVEN: warp t marches ray t.  cow_render_rays of 2^17 rays or
  * more that are mostly alike their neighbours (a camera's rays) are marched one
- * ray per thread in the given order.  Outputs are written at each ray's own
- * index either way and each ray's values are the same; gradient sums change
- * only by the order of their FP32 reductions.  The order costs a key pass, a scan and a scatter (about
- * 12 bytes a ray and 4 MiB of context scratch).  Errors: INVALID_ARG. */
+ * ray per thread in the given order; a key pass over the rays counts those.
+ * Outputs are written at each ray's own index either way and each ray's values
+ * are the same; gradient sums change only by the order of their FP32
+ * reductions.  The coherent order costs a key pass, a scan and a scatter, about
+ * 12 bytes a ray and 4 MiB of context scratch that grows with the largest call:
+ * a graph captured from a call in that order is valid until a larger call.  The
+ * given order uses no scratch that grows.  Errors: INVALID_ARG. */
 #define COW_RAY_ORDER_GIVEN 0
 #define COW_RAY_ORDER_COHERENT 1
 cow_status cow_set_ray_order(cow_ctx *ctx, int32_t mode);

@@ -565,7 +565,12 @@ void make_ray_recs(const cow_ctx *c, const int32_t *ids, int32_t n, cow::RayRecs
 // The coherent processing order of a ray batch (cow_set_ray_order), or null
 // for the order given: batches below kRayOrderMin rays keep theirs (the sort
 // would cost more than it saves).  The box is the call's blocks' bounding
-// box.  The permutation lives in the context until the next call.
+// box.  The permutation lives in the context until the next call.  alike, when
+// given, receives where the count of alike neighbours will be, or null.  The
+// given order uses no buffer that grows (a graph captured from such a call
+// must outlive every later call's sizes): its count is one of the words
+// allocated with the context, each call's the next one, so that calls on
+// several streams do not share it.
 constexpr int64_t kRayOrderMin = 8192;
 
 cow_status ray_order(cow_ctx *c, const float *o, const float *d, int64_t n, const int32_t *ids, int32_t n_ids,
@@ -573,13 +578,7 @@ cow_status ray_order(cow_ctx *c, const float *o, const float *d, int64_t n, cons
     *perm = nullptr;
     if (alike) *alike = nullptr;
     const bool sort = c->ray_order == COW_RAY_ORDER_COHERENT && n >= kRayOrderMin;
-    bool count = alike && n >= cow::kRaysAlikeMin;
-    if (count && !sort && (c->ray_keys.cap < (size_t)n * sizeof(uint32_t) || !c->ray_hist.cap)) {
-        // the given order needs no scratch otherwise: none is allocated inside a capture
-        cudaStreamCaptureStatus cs = cudaStreamCaptureStatusNone;
-        if (cudaStreamIsCapturing(st, &cs) != cudaSuccess) cudaGetLastError();
-        if (cs != cudaStreamCaptureStatusNone) count = false;
-    }
+    const bool count = alike && n >= cow::kRaysAlikeMin;
     if (!(sort || count) || n > 0x7fffffff) return COW_OK;
     float lo[3] = {3.0e38f, 3.0e38f, 3.0e38f}, hi[3] = {-3.0e38f, -3.0e38f, -3.0e38f};
     for (int32_t k = 0; k < n_ids; k++) {
@@ -589,12 +588,18 @@ cow_status ray_order(cow_ctx *c, const float *o, const float *d, int64_t n, cons
             hi[a] = std::max(hi[a], b.hi[a]);
         }
     }
+    if (!sort) {
+        uint32_t *n_alike = c->d_err + cowi::kCtxAlike + c->alike_word++ % cowi::kCtxAlikeWords;
+        COW_CUDA(cow::launch_count_alike(o, d, n, lo, hi, n_alike, st));
+        *alike = n_alike;
+        return COW_OK;
+    }
     COW_CUDA(c->ray_keys.reserve((size_t)n * sizeof(uint32_t)));
     COW_CUDA(c->ray_hist.reserve((size_t)cow::kRayOrderHistWords * sizeof(uint32_t)));
-    if (sort) COW_CUDA(c->ray_perm.reserve((size_t)n * sizeof(int32_t)));
+    COW_CUDA(c->ray_perm.reserve((size_t)n * sizeof(int32_t)));
     COW_CUDA(cow::launch_ray_order(o, d, n, lo, hi, (uint32_t *)c->ray_keys.p, (uint32_t *)c->ray_hist.p,
-                                   sort ? (int32_t *)c->ray_perm.p : nullptr, st));
-    if (sort) *perm = (const int32_t *)c->ray_perm.p;
+                                   (int32_t *)c->ray_perm.p, st));
+    *perm = (const int32_t *)c->ray_perm.p;
     if (count) *alike = (const uint32_t *)c->ray_hist.p + cow::kRayOrderAlike;
     return COW_OK;
 }

@@ -125,7 +125,11 @@ inline double focal_length(int32_t H, double fov_y_deg) {
     return (0.5 * (double)H) / tan(0.5 * fov_y_deg * M_PI / 180.0);
 }
 
-constexpr int kCtxLossParts = 32, kCtxWords = kCtxLossParts + cow::kOpacityMaxCtas;
+// Words allocated with a context: the error word, the counts of alike rays of
+// given-order ray batches (calls take them in turn), the opacity loss's
+// partial sums.
+constexpr int kCtxAlike = 16, kCtxAlikeWords = 16, kCtxLossParts = kCtxAlike + kCtxAlikeWords;
+constexpr int kCtxWords = kCtxLossParts + cow::kOpacityMaxCtas;
 
 }  // namespace cowi
 
@@ -172,7 +176,8 @@ struct cow_ctx {
     uint32_t test_flags = 0, wait_polls = 0;  // cow_set_test_hooks
     std::vector<cowi::BlockHost> blocks;
     std::vector<cow::BlockRec> recs;  // block records (kernels receive copies by value)
-    unsigned *d_err = nullptr;  // kCtxWords words: the error word, at kCtxLossParts the opacity loss's partial sums
+    unsigned *d_err = nullptr;  // kCtxWords words, the error word first
+    unsigned alike_word = 0;    // the next of the kCtxAlikeWords counts
     float *d_mlp = nullptr;
     cowi::DevBuf views, out_rgb, out_aux, out_nsamp;
     cowi::DevBuf gptrs, partials;  // backward: per-block gradient pointers, per-CTA MLP-gradient rows

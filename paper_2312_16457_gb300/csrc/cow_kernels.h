@@ -59,8 +59,8 @@ cudaError_t launch_march_rays(const MarchArgs &a, const RayRecs &rr, cudaStream_
 // marches, grouping rays by the cells of their entry into the box [lo, hi]
 // and their exit from it.  keys: n scratch words; hist: kRayOrderHistWords
 // words (the bins; at kRayOrderAlike the count of rays whose key is the next
-// ray's; the totals of the scan's blocks of 1024 bins).  perm may be null: the
-// count alone.
+// ray's; the totals of the scan's blocks of 1024 bins).  launch_count_alike:
+// the count alone, in its own word.
 constexpr int kRayOrderKeyBits = 20;
 constexpr int kRayOrderBins = 1 << kRayOrderKeyBits;
 constexpr int kRayOrderAlike = kRayOrderBins;
@@ -69,6 +69,8 @@ constexpr int kRayOrderHistWords = kRayOrderBins + 32 + kRayOrderBins / 1024;
 constexpr int64_t kRaysAlikeMin = 1 << 17;
 cudaError_t launch_ray_order(const float *o, const float *d, int64_t n, const float lo[3], const float hi[3],
                              uint32_t *keys, uint32_t *hist, int32_t *perm, cudaStream_t st);
+cudaError_t launch_count_alike(const float *o, const float *d, int64_t n, const float lo[3], const float hi[3],
+                               uint32_t *n_alike, cudaStream_t st);
 // Block-parallel form: per-block partials of a ray batch (8 floats per ray
 // and block, in the order of rr), and K2, their near-to-far "over" with the
 // deferred MLP (Eq. 12-13, Eq. 3).

@@ -37,9 +37,19 @@ __device__ __forceinline__ uint32_t cell_of(float x, float lo, float inv_ext, in
     return (uint32_t)q;
 }
 
-// axes: the axis of every step, two bits each, first step lowest
-__global__ void k_ray_keys(const float *__restrict__ o, const float *__restrict__ d, int64_t n, float3 lo, float3 hi,
-                           uint32_t axes, int3 bits, uint32_t *__restrict__ keys, uint32_t *__restrict__ hist, bool sort) {
+// What the keys are made of: the box, the axis of every step (two bits each,
+// first step lowest) and the steps of each axis.
+struct KeyGrid {
+    float3 lo, hi;
+    uint32_t axes;
+    int3 bits;
+};
+
+// kSort: the keys and their histogram for the order; the count either way.
+template <bool kSort>
+__global__ void k_ray_keys(const float *__restrict__ o, const float *__restrict__ d, int64_t n, KeyGrid kg,
+                           uint32_t *__restrict__ keys, uint32_t *__restrict__ hist, uint32_t *__restrict__ n_alike) {
+    const float3 lo = kg.lo, hi = kg.hi;
     const float3 inv = make_float3(1.f / fmaxf(hi.x - lo.x, 1e-30f), 1.f / fmaxf(hi.y - lo.y, 1e-30f),
                                    1.f / fmaxf(hi.z - lo.z, 1e-30f));
     unsigned same = 0;  // of this warp's rays: those whose key is the next ray's
@@ -61,7 +71,7 @@ __global__ void k_ray_keys(const float *__restrict__ o, const float *__restrict_
             }
             tf = fmaxf(tf, tn);
             const float iv[3] = {inv.x, inv.y, inv.z};
-            const int nb[3] = {bits.x, bits.y, bits.z};
+            const int nb[3] = {kg.bits.x, kg.bits.y, kg.bits.z};
             uint32_t in[3], out[3];  // the axis' cells, the next bit on top
 #pragma unroll
             for (int a = 0; a < 3; a++) {
@@ -73,20 +83,22 @@ __global__ void k_ray_keys(const float *__restrict__ o, const float *__restrict_
             for (int s = 0; s < kSteps; s++) {
 #pragma unroll
                 for (int a = 0; a < 3; a++) {
-                    if ((int)((axes >> (2 * s)) & 3u) != a) continue;  // uniform
+                    if ((int)((kg.axes >> (2 * s)) & 3u) != a) continue;  // uniform
                     key = (key << 2) | (in[a] >> 31 << 1) | (out[a] >> 31);
                     in[a] <<= 1;
                     out[a] <<= 1;
                 }
             }
-            keys[i] = key;
-            if (sort) atomicAdd(hist + key, 1u);
+            if (kSort) {
+                keys[i] = key;
+                atomicAdd(hist + key, 1u);
+            }
         }
         const uint32_t next = __shfl_down_sync(0xffffffffu, key, 1);
         const bool pair = i + 1 < n && (threadIdx.x & 31) != 31 && next == key;
         same += __popc(__ballot_sync(0xffffffffu, pair));
     }
-    if ((threadIdx.x & 31) == 0 && same) atomicAdd(hist + kRayOrderAlike, same);
+    if ((threadIdx.x & 31) == 0 && same) atomicAdd(n_alike, same);
 }
 
 // Exclusive prefix sum of the kRayOrderBins counts in two levels: every CTA
@@ -142,19 +154,8 @@ __global__ void k_ray_scatter(const uint32_t *__restrict__ keys, int64_t n, uint
     }
 }
 
-}  // namespace
-
-cudaError_t launch_ray_order(const float *o, const float *d, int64_t n, const float lo[3], const float hi[3],
-                             uint32_t *keys, uint32_t *hist, int32_t *perm, cudaStream_t st) {
-    static_assert(kRayOrderBins == kScanBlocks * kScanThreads && kScanBlocks <= 1024 && kScanBlocks % 32 == 0,
-                  "two-level scan shape");
-    static_assert(kRayOrderHistWords == kRayOrderBins + 32 + kScanBlocks && kRayOrderAlike == kRayOrderBins,
-                  "histogram scratch: bins, the count of alike neighbours, block totals");
-    if (n <= 0 || n > 0x7fffffff) return cudaErrorInvalidValue;
-    cudaError_t e = cudaMemsetAsync(hist, 0, (kRayOrderAlike + 1) * sizeof(uint32_t), st);
-    if (e != cudaSuccess) return e;
-    uint32_t *sums = hist + kRayOrderBins + 32;
-    // the steps go to the axis whose cells are the longest: near cubic cells
+// Every step halves the longest edge of the cells: near cubic cells.
+KeyGrid key_grid(const float lo[3], const float hi[3]) {
     uint32_t axes = 0;
     int nb[3] = {0, 0, 0};
     float ext[3];
@@ -167,13 +168,37 @@ cudaError_t launch_ray_order(const float *o, const float *d, int64_t n, const fl
         nb[a]++;
         ext[a] *= 0.5f;
     }
-    const int grid = (int)std::min<int64_t>((n + 255) / 256, 152 * 16);
-    k_ray_keys<<<grid, 256, 0, st>>>(o, d, n, make_float3(lo[0], lo[1], lo[2]), make_float3(hi[0], hi[1], hi[2]), axes,
-                                     make_int3(nb[0], nb[1], nb[2]), keys, hist, perm != nullptr);
-    if (!perm) return cudaGetLastError();
+    return {make_float3(lo[0], lo[1], lo[2]), make_float3(hi[0], hi[1], hi[2]), axes, make_int3(nb[0], nb[1], nb[2])};
+}
+
+int key_blocks(int64_t n) { return (int)std::min<int64_t>((n + 255) / 256, 152 * 16); }
+
+}  // namespace
+
+cudaError_t launch_ray_order(const float *o, const float *d, int64_t n, const float lo[3], const float hi[3],
+                             uint32_t *keys, uint32_t *hist, int32_t *perm, cudaStream_t st) {
+    static_assert(kRayOrderBins == kScanBlocks * kScanThreads && kScanBlocks <= 1024 && kScanBlocks % 32 == 0,
+                  "two-level scan shape");
+    static_assert(kRayOrderHistWords == kRayOrderBins + 32 + kScanBlocks && kRayOrderAlike == kRayOrderBins,
+                  "histogram scratch: bins, the count of alike neighbours, block totals");
+    if (n <= 0 || n > 0x7fffffff) return cudaErrorInvalidValue;
+    cudaError_t e = cudaMemsetAsync(hist, 0, (kRayOrderAlike + 1) * sizeof(uint32_t), st);
+    if (e != cudaSuccess) return e;
+    uint32_t *sums = hist + kRayOrderBins + 32;
+    const int grid = key_blocks(n);
+    k_ray_keys<true><<<grid, 256, 0, st>>>(o, d, n, key_grid(lo, hi), keys, hist, hist + kRayOrderAlike);
     k_scan_local<<<kScanBlocks, kScanThreads, 0, st>>>(hist, sums);
     k_scan_sums<<<1, kScanBlocks, 0, st>>>(sums);
     k_ray_scatter<<<grid, 256, 0, st>>>(keys, n, hist, sums, perm);
+    return cudaGetLastError();
+}
+
+cudaError_t launch_count_alike(const float *o, const float *d, int64_t n, const float lo[3], const float hi[3],
+                               uint32_t *n_alike, cudaStream_t st) {
+    if (n <= 0 || n > 0x7fffffff) return cudaErrorInvalidValue;
+    cudaError_t e = cudaMemsetAsync(n_alike, 0, sizeof(uint32_t), st);
+    if (e != cudaSuccess) return e;
+    k_ray_keys<false><<<key_blocks(n), 256, 0, st>>>(o, d, n, key_grid(lo, hi), nullptr, nullptr, n_alike);
     return cudaGetLastError();
 }
 
