@@ -340,12 +340,11 @@ __device__ __forceinline__ bool remarch_block(BwdScratch &bs, const BlockRec &b,
         T = __shfl_sync(kFullMask, T, 0);
         bool more = true;
         int used = n;
-        if (T < ert_eps) {  // the ray ends in this chunk
-            more = false;
+        if (!(T >= ert_eps)) {  // the ray ends in this chunk, perhaps in front of a NaN
             float Ts = s.T;
-            for (used = 0; used < n;) {
+            for (used = 0; used < n && more;) {
                 Ts *= ws.row[7][used++];
-                if (Ts < ert_eps) break;
+                more = !(Ts < ert_eps);
             }
         }
         s.T = T;

@@ -201,8 +201,7 @@ __device__ __forceinline__ bool composite_chunk(WarpScratch &ws, int n, float e,
     }
     bool more = true;
     int used = n;
-    if (T < ert_eps) {  // the ray ends in this chunk: again, up to there
-        more = false;
+    if (!(T >= ert_eps)) {  // the ray ends in this chunk, perhaps in front of a NaN: again, up to there
         T = s.T;
         acc = s.acc;
         const float *er = ws.row[7], *xr = ws.row[lane & 7];
@@ -211,7 +210,10 @@ __device__ __forceinline__ bool composite_chunk(WarpScratch &ws, int n, float e,
             acc = fmaf(T * (1.f - ev), xr[used], acc);
             T *= ev;
             used++;
-            if (T < ert_eps) break;
+            if (T < ert_eps) {
+                more = false;
+                break;
+            }
         }
     }
     __syncwarp();
