@@ -664,9 +664,10 @@ cow_status cow_set_schedule(cow_ctx *ctx, int32_t schedule);
  * by a counting sort on the device -- so that the rays on the chip at one time
  * gather neighbouring texels and share them in L2 (measured on 2^20 random rays
  * over 2x2 blocks of 128^3 / 512^2 FP32 features: forward 39.9 -> 28.3 ms).
- * COW_RAY_ORDER_GIVEN: warp t marches ray t.  cow_render_rays of 2^17 rays or
- * more that are mostly alike their neighbours (a camera's rays) are marched one
- * ray per thread in the given order; a key pass over the rays counts those.
+ * COW_RAY_ORDER_GIVEN: warp t marches ray t.  Calls of 2^17 rays or more that
+ * are mostly alike their neighbours (a camera's rays) are marched one ray per
+ * thread in the given order, but for the backwards and the opacity gradient; a
+ * key pass over the rays counts the alike ones.
  * Outputs are written at each ray's own index either way and each ray's values
  * are the same; gradient sums change only by the order of their FP32
  * reductions.  The coherent order costs a key pass, a scan and a scatter, about
@@ -699,6 +700,15 @@ cow_status cow_tune_schedule(cow_ctx *ctx, const cow_camera *cams, int32_t n_vie
  * this context (COW_ERR_DEVICE_ASSERT or COW_ERR_TIMEOUT); clears it. */
 cow_status cow_sync_check(cow_ctx *ctx, void *stream);
 
+/* Which form the last cow_render, cow_render_rays*, cow_render_partials or
+ * cow_opacity_loss call of the context took (no counterpart in the paper): one
+ * ray per warp or one ray per thread.  The form shows in the time only.  Where
+ * the device decides (mostly alike rays), waits for the stream.  Errors:
+ * INVALID_ARG (null argument, no such call yet), CUDA. */
+#define COW_FORM_WARP 0
+#define COW_FORM_THREAD 1
+cow_status cow_last_form(cow_ctx *ctx, void *stream, int32_t *out_form);
+
 /* Test hook (no counterpart in the paper): lets a test drive the bounded
  * device-side waits to their time-out without faulting anything.  The
  * kernels that stage a view's block records into shared memory with a TMA
@@ -711,6 +721,10 @@ cow_status cow_sync_check(cow_ctx *ctx, void *stream);
  * writing their pixels, and the context stays usable.  Production callers
  * never call this (flags 0, wait_polls 0).  Errors: INVALID_ARG. */
 #define COW_TEST_SKIP_RECORD_COPY 1u
+/* The form of the marches that choose one (COW_SCHED_THREAD_CONST views and
+ * ray batches without a backward) in place of the size rules. */
+#define COW_TEST_THREAD_FORM 2u
+#define COW_TEST_WARP_FORM 4u
 cow_status cow_set_test_hooks(cow_ctx *ctx, uint32_t flags, uint32_t wait_polls);
 
 /* Copy out a block's occupancy bits (ceil(ncell/32) words, cell index

@@ -46,7 +46,7 @@ EXPORTS = ["cow_load_blocks", "cow_load_blocks_ex", "cow_save_scene", "cow_load_
            "cow_batch_set_views", "cow_batch_render", "cow_batch_set_config", "cow_batch_tune",
            "cow_batch_last_groups", "cow_batch_set_run_fraction", "cow_batch_set_records", "cow_batch_get_config",
            "cow_batch_set_schedule", "cow_batch_get_schedule", "cow_set_ray_order", "cow_render_rays_block_state",
-           "cow_render_backward_block_mlps_state", "cow_tune_schedule", "cow_last_error",
+           "cow_render_backward_block_mlps_state", "cow_tune_schedule", "cow_last_form", "cow_last_error",
            "cow_version"]
 SCHEDULES = {"warp": 0, "thread": 1, "thread_const": 2}
 
@@ -136,6 +136,7 @@ def lib():
             "cow_batch_get_config": [P, P, P, P],
             "cow_batch_set_schedule": [P, i32],
             "cow_set_ray_order": [P, i32],
+            "cow_last_form": [P, P, P],
             "cow_render_rays_block_state": [P, P, P, i64, P, i32, P, P, P],
             "cow_render_backward_block_mlps_state": [P, P, P, i64, P, i32, P, P, P, P, P, P],
             "cow_batch_get_schedule": [P, P],
@@ -513,9 +514,19 @@ class Context:
         """0: raster tile order; k > 0: vertical strips of k tile columns."""
         _check(lib().cow_set_tile_order(self._ctx, int(strip_tiles)))
 
-    def set_test_hooks(self, skip_record_copy: bool = False, wait_polls: int = 0):
-        """Tests of the bounded device waits (cow_set_test_hooks)."""
-        _check(lib().cow_set_test_hooks(self._ctx, 1 if skip_record_copy else 0, int(wait_polls)))
+    FORMS = {"warp": 0, "thread": 1}
+
+    def last_form(self, stream=None) -> str:
+        """"warp" or "thread": the form of the last march (cow_last_form)."""
+        k = C.c_int32()
+        _check(lib().cow_last_form(self._ctx, _stream_ptr(stream), C.byref(k)))
+        return {v: n for n, v in self.FORMS.items()}[k.value]
+
+    def set_test_hooks(self, skip_record_copy: bool = False, wait_polls: int = 0, form: Optional[str] = None):
+        """Tests of the bounded device waits and of one march form
+        (cow_set_test_hooks)."""
+        flags = (1 if skip_record_copy else 0) | {None: 0, "thread": 2, "warp": 4}[form]
+        _check(lib().cow_set_test_hooks(self._ctx, flags, int(wait_polls)))
 
     def sync_check(self, stream=None):
         _check(lib().cow_sync_check(self._ctx, _stream_ptr(stream)))

@@ -588,7 +588,8 @@ __global__ void __launch_bounds__(kBwdThreads, COW_REG_MIN_BLOCKS) k_opacity(con
     const int lane = threadIdx.x & 31;
     float term = 0.f;
     const float scale = a.weight / (float)a.n_rays, eps = 1e-6f;
-    for (int64_t ray = first_ray(); ray < a.n_rays; ray += (int64_t)gridDim.x * kBwdWarps) {
+    const int64_t n_rays = rays_alike(a) ? 0 : a.n_rays;  // alike: k_opacity_t has them
+    for (int64_t ray = first_ray(); ray < n_rays; ray += (int64_t)gridDim.x * kBwdWarps) {
         float o[3], d[3], inv_d[3], omax;
         const int64_t r = load_ray_warp(a, ray, o, d);
         ray_setup(d, o, inv_d, omax);
@@ -643,11 +644,70 @@ __global__ void __launch_bounds__(kBwdThreads, COW_REG_MIN_BLOCKS) k_opacity(con
     if (threadIdx.x == 0) a.loss_parts[blockIdx.x] = term;
 }
 
+// The same, one ray per thread (ray_form in cow_api.cu), every sample
+// scattered by its own thread; the loss's parts behind k_opacity's.
+template <int DT>
+__global__ void __launch_bounds__(kBwdThreads, COW_REG_MIN_BLOCKS) k_opacity_t(const __grid_constant__ RegArgs a,
+                                                                            const __grid_constant__ RayRecs rr) {
+    float term = 0.f;
+    const float scale = a.weight / (float)a.n_rays, eps = 1e-6f;
+    bool given;
+    const int64_t n_rays = thread_form(a, given) ? a.n_rays : 0;
+    for (int64_t ray = (int64_t)blockIdx.x * kBwdThreads + threadIdx.x; ray < n_rays;
+         ray += (int64_t)gridDim.x * kBwdThreads) {
+        float o[3], d[3], inv_d[3], omax;
+        const int64_t r = load_ray(a, ray, given, o, d);
+        ray_setup(d, o, inv_d, omax);
+        int order[kMaxRayIds];
+        const int n = sort_blocks_for_ray(rr, o, order);
+        for (int k = 0; k < n; k++) {
+            const int pos = order[k], id = rr.id[pos];
+            const BlockRec &b = rr.r[pos];
+            float T = 1.f;
+            if (a.block_T) {
+                T = __ldg(a.block_T + r * rr.n + pos);
+                if (T < 0.f) continue;
+            } else {
+                int nk = 0;
+                DepthSum tau;
+                BrickCache bc;
+                for_each_sample(b, o, d, inv_d, omax, a.err,
+                                [&](const float *, const float rel[3], const float g[3], float delta) {
+                    float2 f2[4];
+                    accumulate_sample<DT>(b, rel, g, f2, &bc);
+                    tau.add(expf(f2[0].x) * delta);
+                    nk++;
+                    return true;
+                });
+                if (nk == 0) continue;
+                T = tau.transmittance();
+            }
+            const float a_raw = 1.f - T;
+            const float al = fminf(fmaxf(a_raw, eps), 1.f - eps);
+            term -= scale * (al * logf(al) + (1.f - al) * log1pf(-al));
+            if (!a.grad_grid || !(a_raw > eps && a_raw < 1.f - eps)) continue;
+            const float ga = -scale * (logf(al) - log1pf(-al));
+            float *const gp[3] = {a.grad_planes[3 * id], a.grad_planes[3 * id + 1], a.grad_planes[3 * id + 2]};
+            BrickCache bc;
+            for_each_sample(b, o, d, inv_d, omax, a.err,
+                            [&](const float *, const float rel[3], const float g[3], float delta) {
+                float2 f2[4];
+                accumulate_sample<DT>(b, rel, g, f2, &bc);
+                scatter_ch0(b, a.grad_grid[id], gp, rel, g, ga * expf(f2[0].x) * delta * T);
+                return true;
+            });
+        }
+    }
+    term = cta_sum(term);
+    if (threadIdx.x == 0) a.loss_parts[kOpacityMaxCtas + blockIdx.x] = term;
+}
+
 // *loss += the CTAs' sums (in a fixed order: thousands of additions to one
 // float would cost its last bits)
-__global__ void __launch_bounds__(1024) k_add_parts(const float *__restrict__ parts, int n, float *loss) {
+__global__ void __launch_bounds__(1024) k_add_parts(const float *__restrict__ parts, int nw, int nt, float *loss) {
     float v = 0.f;
-    for (int k = threadIdx.x; k < n; k += 1024) v += parts[k];
+    for (int k = threadIdx.x; k < nw; k += 1024) v += parts[k];
+    for (int k = threadIdx.x; k < nt; k += 1024) v += parts[kOpacityMaxCtas + k];
     v = cta_sum(v);
     if (threadIdx.x == 0) atomicAdd(loss, v);
 }
@@ -1022,16 +1082,20 @@ cudaError_t launch_sparsity(const RegArgs &a, const RayRecs &rr, cudaStream_t st
 
 cudaError_t launch_opacity(const RegArgs &a, const RayRecs &rr, cudaStream_t st) {
     if (a.n_rays <= 0) return cudaSuccess;
-    // one ray per warp; beyond kOpacityMaxCtas CTAs (8 waves) one ray after another
-    const unsigned nw = (unsigned)std::min<int64_t>((a.n_rays + kBwdWarps - 1) / kBwdWarps, kOpacityMaxCtas);
-    {
-        const cudaError_t e_ = dispatch_dt(a.dtype, [&](auto D) {
-            k_opacity<decltype(D)::value><<<nw, kBwdThreads, 0, st>>>(a, rr);
-            return cudaSuccess;
-        });
-        if (e_ != cudaSuccess) return e_;
-    }
-    if (a.loss) k_add_parts<<<1, 1024, 0, st>>>(a.loss_parts, (int)nw, a.loss);
+    // a ray per warp or per thread; beyond kOpacityMaxCtas CTAs (8 waves) one ray after another
+    const auto ctas = [&](int rays) {
+        return (unsigned)std::min<int64_t>((a.n_rays + rays - 1) / rays, kOpacityMaxCtas);
+    };
+    // as launch_rays_dt: with a count of alike rays both are launched
+    const unsigned nw = a.form == kFormWarp ? ctas(kBwdWarps) : 0;
+    const unsigned nt = a.form == kFormThread || a.ray_alike ? ctas(kBwdThreads) : 0;
+    const cudaError_t e_ = dispatch_dt(a.dtype, [&](auto D) {
+        if (nt) k_opacity_t<decltype(D)::value><<<nt, kBwdThreads, 0, st>>>(a, rr);
+        if (nw) k_opacity<decltype(D)::value><<<nw, kBwdThreads, 0, st>>>(a, rr);
+        return cudaSuccess;
+    });
+    if (e_ != cudaSuccess) return e_;
+    if (a.loss) k_add_parts<<<1, 1024, 0, st>>>(a.loss_parts, (int)nw, (int)nt, a.loss);
     return cudaGetLastError();
 }
 
@@ -1042,7 +1106,7 @@ cudaError_t launch_adam(float *p, const float *g, float *m, float *v, int64_t n,
     const bool vec = !(((uintptr_t)p | (uintptr_t)g | (uintptr_t)m | (uintptr_t)v) & 15u);
     const int64_t n4 = vec ? n / 4 : 0;
     int64_t blocks = ((vec ? n4 : n) + 255) / 256;
-    if (blocks > 152 * 32) blocks = 152 * 32;
+    if (blocks > kSms * 32) blocks = kSms * 32;
     if (blocks < 1) blocks = 1;
     k_adam<<<(int)blocks, 256, 0, st>>>(p, g, m, v, n, n4, AdamArgs{lr, b1, b2, eps, bc1, bc2});
     return cudaGetLastError();
@@ -1057,7 +1121,7 @@ cudaError_t launch_mse_grad(const float *rgb, const float *tgt, int64_t n, float
     // one CTA of 32 warps per SM at most: every CTA adds its part to the loss, and
     // the 2432 additions of 3.1 M values at 256 threads a CTA cost it 1.5e-6
     int64_t blocks = (n + 1023) / 1024;
-    if (blocks > 152) blocks = 152;
+    if (blocks > kSms) blocks = kSms;
     k_mse_grad<<<(int)blocks, 1024, 0, st>>>(rgb, tgt, n, 1.0f / (float)n, grad, loss);
     return cudaGetLastError();
 }

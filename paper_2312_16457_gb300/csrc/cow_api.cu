@@ -565,8 +565,8 @@ void make_ray_recs(const cow_ctx *c, const int32_t *ids, int32_t n, cow::RayRecs
 // The coherent processing order of a ray batch (cow_set_ray_order), or null
 // for the order given: batches below kRayOrderMin rays keep theirs (the sort
 // would cost more than it saves).  The box is the call's blocks' bounding
-// box.  The permutation lives in the context until the next call.  alike, when
-// given, receives where the count of alike neighbours will be, or null.  The
+// box.  The permutation lives in the context until the next call.  With
+// `count`, *alike receives where the count of alike neighbours will be.  The
 // given order uses no buffer that grows (a graph captured from such a call
 // must outlive every later call's sizes): its count is one of the words
 // allocated with the context, each call's the next one, so that calls on
@@ -574,11 +574,10 @@ void make_ray_recs(const cow_ctx *c, const int32_t *ids, int32_t n, cow::RayRecs
 constexpr int64_t kRayOrderMin = 8192;
 
 cow_status ray_order(cow_ctx *c, const float *o, const float *d, int64_t n, const int32_t *ids, int32_t n_ids,
-                     cudaStream_t st, const int32_t **perm, const uint32_t **alike = nullptr) {
+                     cudaStream_t st, const int32_t **perm, bool count = false, const uint32_t **alike = nullptr) {
     *perm = nullptr;
     if (alike) *alike = nullptr;
     const bool sort = c->ray_order == COW_RAY_ORDER_COHERENT && n >= kRayOrderMin;
-    const bool count = alike && n >= cow::kRaysAlikeMin;
     if (!(sort || count) || n > 0x7fffffff) return COW_OK;
     float lo[3] = {3.0e38f, 3.0e38f, 3.0e38f}, hi[3] = {-3.0e38f, -3.0e38f, -3.0e38f};
     for (int32_t k = 0; k < n_ids; k++) {
@@ -602,6 +601,52 @@ cow_status ray_order(cow_ctx *c, const float *o, const float *d, int64_t n, cons
     *perm = (const int32_t *)c->ray_perm.p;
     if (count) *alike = (const uint32_t *)c->ray_hist.p + cow::kRayOrderAlike;
     return COW_OK;
+}
+
+// --- one ray per warp or one ray per thread ---------------------------------
+// One ray per warp takes a ray's samples 32 at a time: the call is not held up
+// by its longest ray's chain of gathers, and random rays do not diverge.  One
+// ray per thread costs less a ray (no queue, no ordered composite, an MLP a
+// lane), shares lines between the rays of a warp where they are alike, and
+// walks the points of an unbounded block once a lane instead of once a warp.
+
+int32_t forced_form(const cow_ctx *c) {
+    return c->test_flags & COW_TEST_THREAD_FORM ? cow::kFormThread : c->test_flags & COW_TEST_WARP_FORM ? cow::kFormWarp : -1;
+}
+
+// Frames of up to kChipRays pixels are marched one ray per warp: one ray per
+// thread then has every ray on the chip at once and takes as long as its longest
+// ray.  Measured (us, thread / warp form): M = 1 block of 64^3 FP32, 128x128
+// 357 / 98, 320x240 389 / 337, 400x300 488 / 525; 4x4 blocks of 128^3 BF16,
+// 96x54 2585 / 125, 320x240 2223 / 1382, 400x300 2286 / 2113, 480x360 2662 /
+// 2996; three-level city BF16, 96x54 2985 / 83, 320x240 1885 / 666.
+int32_t view_form(const cow_ctx *c, int64_t n_pix) {
+    if (forced_form(c) >= 0) return forced_form(c);
+    return n_pix <= cow::kChipRays ? cow::kFormWarp : cow::kFormThread;
+}
+
+// What a ray batch is marched for: the outputs of the march, the block-parallel
+// form's partials, the opacity term, the term and its gradient (which marches
+// every block twice), the gradient from the forward's in-block transmittances.
+enum RayCall { kCallMarch, kCallPartials, kCallOpacity, kCallOpacityGrad, kCallOpacityGradT };
+
+// The form of a ray batch.  *count: the device counts the alike rays, and takes
+// the thread form in the given order when it is a camera's.  Measured on 921600
+// camera rays (ms, thread in the given order / warp): 16 blocks of 128^3 FP16,
+// rays 8.7 / 13.4, with in-block transmittances 9.9 / 13.7, partials 9.5 / 12.0,
+// opacity 7.3 / 10.6, with gradients 29.6 / 29.5 and, from the transmittances,
+// 24.2 / 21.1.
+int32_t ray_form(const cow_ctx *c, int64_t n, RayCall call, bool *count) {
+    *count = false;
+    if (forced_form(c) >= 0) return forced_form(c);
+    *count = call != kCallOpacityGrad && call != kCallOpacityGradT && n >= cow::kRaysAlikeMin;
+    return cow::kFormWarp;
+}
+
+void note_form(cow_ctx *c, int32_t form, int64_t n, const uint32_t *alike) {
+    c->last_form = form;
+    c->last_n = n;
+    c->last_alike = alike;
 }
 
 // --- dynamic loading / unloading under a device-memory budget (App. D) -----
@@ -1013,7 +1058,6 @@ cow_status cow_render(cow_ctx *ctx, const cow_camera *cams, int32_t n_views, con
     a.err = ctx->d_err;
     a.test_flags = ctx->test_flags;
     a.wait_polls = ctx->wait_polls;
-    a.n_rays = plan.n_pix;
     if (block_mlp) {
         a.block_mlps = (const float *const *)((unsigned char *)ctx->views.p + vbytes + rbytes);
         a.n_freq = ctx->n_freq;
@@ -1028,13 +1072,15 @@ cow_status cow_render(cow_ctx *ctx, const cow_camera *cams, int32_t n_views, con
         cow::ParamRecs pr;
         std::memset(&pr, 0, sizeof(pr));
         std::copy(vrecs.begin(), vrecs.begin() + n_ids, pr.r);
+        a.form = view_form(ctx, plan.n_pix);
         COW_CUDA(cow::launch_march_views(a, plan.n_tiles, cow::kSchedThreadConst, st, &pr));
     } else {
         // the warp schedule marches bounded blocks only
+        a.form = ctx->schedule == COW_SCHED_WARP && !any_unbounded ? cow::kFormWarp : cow::kFormThread;
         COW_CUDA(cow::launch_march_views(a, plan.n_tiles,
-                                         ctx->schedule == COW_SCHED_WARP && !any_unbounded ? cow::kSchedWarp
-                                                                                           : cow::kSchedThread, st));
+                                         a.form == cow::kFormWarp ? cow::kSchedWarp : cow::kSchedThread, st));
     }
+    note_form(ctx, a.form, 0, nullptr);
     if ((rc = note_use_impl(ctx, ids, n_ids, st)) != COW_OK) return rc;
     if (h_rgb) COW_CUDA(cudaMemcpyAsync(out_rgb, rgb, (size_t)plan.n_pix * 12, cudaMemcpyDeviceToHost, st));
     if (h_aux) COW_CUDA(cudaMemcpyAsync(out_aux, aux, (size_t)plan.n_pix * 32, cudaMemcpyDeviceToHost, st));
@@ -1099,12 +1145,13 @@ static cow_status render_rays_impl(cow_ctx *ctx, const float *o, const float *d,
         a.block_mlp_stride = ctx->block_mlp_nparam;
         a.n_freq = ctx->n_freq;
     }
-    if ((rc = ray_order(ctx, o, d, n_rays, ids, n_ids, st, &a.ray_perm,
-                        out_block_T || out_block_state ? nullptr : &a.ray_alike)) != COW_OK)
-        return rc;
+    bool count;
+    a.form = ray_form(ctx, n_rays, kCallMarch, &count);
+    if ((rc = ray_order(ctx, o, d, n_rays, ids, n_ids, st, &a.ray_perm, count, &a.ray_alike)) != COW_OK) return rc;
     cow::RayRecs rr;
     make_ray_recs(ctx, ids, n_ids, rr);
     COW_CUDA(cow::launch_march_rays(a, rr, st));
+    note_form(ctx, a.form, n_rays, a.ray_alike);
     if ((rc = note_use_impl(ctx, ids, n_ids, st)) != COW_OK) return rc;
     if (h_rgb) COW_CUDA(cudaMemcpyAsync(out_rgb, rgb, (size_t)n_rays * 12, cudaMemcpyDeviceToHost, st));
     if (h_aux) COW_CUDA(cudaMemcpyAsync(out_aux, aux, (size_t)n_rays * 32, cudaMemcpyDeviceToHost, st));
@@ -1137,10 +1184,13 @@ cow_status cow_render_partials(cow_ctx *ctx, const float *o, const float *d, int
     a.ray_d = d;
     a.n_rays = n_rays;
     a.out_partials = out_partials;
-    if ((rc = ray_order(ctx, o, d, n_rays, ids, n_ids, st, &a.ray_perm)) != COW_OK) return rc;
+    bool count;
+    a.form = ray_form(ctx, n_rays, kCallPartials, &count);
+    if ((rc = ray_order(ctx, o, d, n_rays, ids, n_ids, st, &a.ray_perm, count, &a.ray_alike)) != COW_OK) return rc;
     cow::RayRecs rr;
     make_ray_recs(ctx, ids, n_ids, rr);
     COW_CUDA(cow::launch_march_partials(a, rr, st));
+    note_form(ctx, a.form, n_rays, a.ray_alike);
     return note_use_impl(ctx, ids, n_ids, st);
 }
 
@@ -1490,10 +1540,14 @@ cow_status cow_opacity_loss(cow_ctx *ctx, const float *o, const float *d, int64_
     a.weight = weight;
     a.block_T = block_T;
     a.loss_parts = (float *)(ctx->d_err + kCtxLossParts);
-    if ((rc = ray_order(ctx, o, d, n_rays, ids, n_ids, st, &a.ray_perm)) != COW_OK) return rc;
+    bool count;
+    const RayCall call = !grad_grid ? kCallOpacity : block_T ? kCallOpacityGradT : kCallOpacityGrad;
+    a.form = ray_form(ctx, n_rays, call, &count);
+    if ((rc = ray_order(ctx, o, d, n_rays, ids, n_ids, st, &a.ray_perm, count, &a.ray_alike)) != COW_OK) return rc;
     cow::RayRecs rr;
     make_ray_recs(ctx, ids, n_ids, rr);
     COW_CUDA(cow::launch_opacity(a, rr, st));
+    note_form(ctx, a.form, n_rays, a.ray_alike);
     return note_use_impl(ctx, ids, n_ids, st);
 }
 
@@ -1941,9 +1995,26 @@ static_assert(COW_TEST_SKIP_RECORD_COPY == cow::kTestSkipRecordCopy, "test flag 
 cow_status cow_set_test_hooks(cow_ctx *ctx, uint32_t flags, uint32_t wait_polls) {
     g_last_error.clear();
     if (!ctx) return fail(COW_ERR_INVALID_ARG, "null context");
-    if (flags & ~(uint32_t)COW_TEST_SKIP_RECORD_COPY) return fail(COW_ERR_INVALID_ARG, "unknown test flags 0x%x", flags);
+    if (flags & ~(uint32_t)(COW_TEST_SKIP_RECORD_COPY | COW_TEST_THREAD_FORM | COW_TEST_WARP_FORM))
+        return fail(COW_ERR_INVALID_ARG, "unknown test flags 0x%x", flags);
     ctx->test_flags = flags;
     ctx->wait_polls = wait_polls;
+    return COW_OK;
+}
+
+static_assert(COW_FORM_WARP == cow::kFormWarp && COW_FORM_THREAD == cow::kFormThread, "form values");
+
+cow_status cow_last_form(cow_ctx *ctx, void *stream, int32_t *out_form) {
+    g_last_error.clear();
+    if (!ctx || !out_form) return fail(COW_ERR_INVALID_ARG, "null argument");
+    if (ctx->last_form < 0) return fail(COW_ERR_INVALID_ARG, "cow_last_form: no call yet");
+    *out_form = ctx->last_form;
+    if (!ctx->last_alike) return COW_OK;
+    DeviceGuard dg(ctx->device);
+    COW_CUDA(cudaStreamSynchronize((cudaStream_t)stream));
+    uint32_t n = 0;
+    COW_CUDA(cudaMemcpy(&n, ctx->last_alike, sizeof(n), cudaMemcpyDeviceToHost));
+    if (cow::mostly_alike(n, ctx->last_n)) *out_form = COW_FORM_THREAD;
     return COW_OK;
 }
 

@@ -129,7 +129,7 @@ inline double focal_length(int32_t H, double fov_y_deg) {
 // given-order ray batches (calls take them in turn), the opacity loss's
 // partial sums.
 constexpr int kCtxAlike = 16, kCtxAlikeWords = 16, kCtxLossParts = kCtxAlike + kCtxAlikeWords;
-constexpr int kCtxWords = kCtxLossParts + cow::kOpacityMaxCtas;
+constexpr int kCtxWords = kCtxLossParts + 2 * cow::kOpacityMaxCtas;
 
 }  // namespace cowi
 
@@ -178,6 +178,9 @@ struct cow_ctx {
     std::vector<cow::BlockRec> recs;  // block records (kernels receive copies by value)
     unsigned *d_err = nullptr;  // kCtxWords words, the error word first
     unsigned alike_word = 0;    // the next of the kCtxAlikeWords counts
+    int32_t last_form = -1;     // cow_last_form: the last march's form, its rays and its count of alike ones (null: none)
+    int64_t last_n = 0;
+    const uint32_t *last_alike = nullptr;
     float *d_mlp = nullptr;
     cowi::DevBuf views, out_rgb, out_aux, out_nsamp;
     cowi::DevBuf gptrs, partials;  // backward: per-block gradient pointers, per-CTA MLP-gradient rows

@@ -25,7 +25,8 @@ struct MarchArgs {
     unsigned *err;
     const float *ray_o;    // ray mode
     const float *ray_d;
-    int64_t n_rays;        // rays of the call (view mode: pixels)
+    int64_t n_rays;        // ray mode: rays of the call
+    int32_t form;          // kFormWarp or kFormThread
     int32_t smem_recs;     // view mode, thread schedule: block records the launch's shared memory holds
     const float *const *block_mlps;  // view mode, per-block MLPs: weights of record k, parallel to recs
     int32_t n_freq;                  // PE frequencies of the per-block MLPs
@@ -36,11 +37,18 @@ struct MarchArgs {
     uint32_t wait_polls;             // bound on each mbarrier wait (0: the kernel's default)
     float *out_partials;             // block-parallel form: n_rays x n_ids x 8 per-block partials (written)
     const float *in_partials;        // block-parallel form: the same, read by the compositor
-    const int32_t *ray_perm;         // ray mode, may be null: warp t marches ray ray_perm[t] (outputs at the ray's index)
-    const uint32_t *ray_alike;       // ray mode, may be null: rays whose order key is the next ray's
+    const int32_t *ray_perm;         // ray mode, may be null: ray t of the order is ray ray_perm[t] (outputs at the ray's index)
+    const uint32_t *ray_alike;       // ray mode, kFormWarp, may be null: rays whose order key is the next ray's; the
+                                     // device takes kFormThread in the given order when most are (rays_alike)
     float *out_block_state;          // ray mode, per-block MLPs, may be null: n_rays x n_ids x 8, per (ray, block
                                      // at its position in ids) C^k (3), F^k (4), the transmittance in front (-1: no sample)
 };
+
+// The two forms of a march: one ray per warp (march_warp.cuh), one per thread.
+constexpr int32_t kFormWarp = 0, kFormThread = 1;
+constexpr int kSms = 152;  // GB300
+// Rays on the chip at once, one per thread (512 threads per SM).
+constexpr int64_t kChipRays = kSms * 512;
 
 // Test hook of the kernels that stage block records with a TMA bulk copy:
 // the copy is not issued, so the barrier's phase never completes and the
@@ -65,8 +73,10 @@ constexpr int kRayOrderKeyBits = 20;
 constexpr int kRayOrderBins = 1 << kRayOrderKeyBits;
 constexpr int kRayOrderAlike = kRayOrderBins;
 constexpr int kRayOrderHistWords = kRayOrderBins + 32 + kRayOrderBins / 1024;
-// Calls of at least this many rays look at the count (launch_march_rays).
+// Calls of at least this many rays look at the count (ray_form in cow_api.cu).
 constexpr int64_t kRaysAlikeMin = 1 << 17;
+// Whether n of a call's n_rays rays, alike the next one, make it a camera's.
+__host__ __device__ __forceinline__ bool mostly_alike(uint32_t n, int64_t n_rays) { return 4 * (int64_t)n >= 3 * n_rays; }
 cudaError_t launch_ray_order(const float *o, const float *d, int64_t n, const float lo[3], const float hi[3],
                              uint32_t *keys, uint32_t *hist, int32_t *perm, cudaStream_t st);
 cudaError_t launch_count_alike(const float *o, const float *d, int64_t n, const float lo[3], const float hi[3],
@@ -130,13 +140,15 @@ struct RegArgs {                  // the blocks that take part come by value (Ra
     const float *block_T;         // opacity: the forward's n_rays x n_ids in-block transmittances (-1: no
                                   // sample), or null to march every block twice
     float *loss;                  // device float, accumulated (may be null)
-    float *loss_parts;            // opacity: scratch, kOpacityMaxCtas floats
+    float *loss_parts;            // opacity: scratch, 2 kOpacityMaxCtas floats
     float *const *grad_grid;      // device pointer table as in BwdArgs (null: no gradient)
     float *const *grad_planes;
     unsigned *err;
-    const int32_t *ray_perm;      // opacity, may be null: warp t takes ray ray_perm[t]
+    const int32_t *ray_perm;      // opacity, may be null: as in MarchArgs, with
+    const uint32_t *ray_alike;    // opacity, may be null
+    int32_t form;                 // opacity: kFormWarp or kFormThread
 };
-constexpr int kOpacityMaxCtas = 152 * 32;
+constexpr int kOpacityMaxCtas = kSms * 32;
 cudaError_t launch_sparsity(const RegArgs &a, const RayRecs &rr, cudaStream_t st);
 cudaError_t launch_opacity(const RegArgs &a, const RayRecs &rr, cudaStream_t st);
 // threads per CTA of the backward kernels: one MLP-gradient scratch row per

@@ -461,24 +461,39 @@ struct RayState {
     bool done;
 };
 
-// March one ray through one block, updating its state (Eq. 1-2).
+// A sum of optical depths with the rounding of every addition carried along: a
+// block's transmittance is exp(-sum), and one FP32 sum over its samples would
+// be further off than the warp form's 32 short ones.
+struct DepthSum {
+    float s = 0.f, c = 0.f;
+    __device__ __forceinline__ void add(float x) {
+        const float y = __fsub_rn(x, c), t = __fadd_rn(s, y);
+        c = t < 3.0e38f ? __fsub_rn(__fsub_rn(t, s), y) : 0.f;  // infinite: stays so
+        s = t;
+    }
+    __device__ __forceinline__ float transmittance() const { return expf(-s); }
+};
+
+// March one ray through one block, updating its state (Eq. 1-2) and, when
+// given, the block's own optical depth (Eq. 11).
 template <int DT>
 __device__ __forceinline__ void march_block(const BlockRec &b, const float o[3], const float d[3],
                                             const float inv_d[3], float omax, float ert_eps, RayState &s,
-                                            unsigned *err) {
+                                            unsigned *err, DepthSum *depth = nullptr) {
     BrickCache bc;
     const bool more = for_each_sample(b, o, d, inv_d, omax, err, [&](const float *, const float rel[3], const float g[3], float dt) {
         float2 f2[4];
         accumulate_sample<DT>(b, rel, g, f2, &bc);
         const float f[8] = {f2[0].x, f2[0].y, f2[1].x, f2[1].y, f2[2].x, f2[2].y, f2[3].x, f2[3].y};
-        const float sigma = __expf(f[0]);
-        const float e = __expf(-sigma * dt);
+        const float sd = __expf(f[0]) * dt;
+        const float e = __expf(-sd);
         const float w = s.T * (1.f - e);
 #pragma unroll
         for (int c = 0; c < 3; c++) s.Cd[c] = fmaf(w, sigmoidf_fast(f[1 + c]), s.Cd[c]);
 #pragma unroll
         for (int c = 0; c < 4; c++) s.F[c] = fmaf(w, sigmoidf_fast(f[4 + c]), s.F[c]);
         s.T *= e;
+        if (depth) depth->add(sd);
         s.nsamp++;
         return !(s.T < ert_eps);
     });

@@ -82,16 +82,23 @@ __device__ __forceinline__ int view_of_tile(const MarchArgs &a, int tile) {
 // T carries the product of the blocks' 1 - alpha^k.  Early termination uses
 // the ray's total transmittance: inside block k it stops once
 // T_k < ert_eps / T.  rec_at(k) / mlp_at(k): the k-th block's record and
-// MLP weights in near-to-far order.
-template <int DT, class RecAt, class MlpAt>
+// MLP weights in near-to-far order; state(k): where the k-th block's state
+// goes (a.out_block_state, ray mode), or null.
+template <int DT, class RecAt, class MlpAt, class StateAt>
 __device__ __forceinline__ void blend_blocks(const MarchArgs &a, int n_blk, RecAt rec_at, MlpAt mlp_at,
-                                             const float o[3], const float d[3], const float inv_d[3], float omax,
-                                             int64_t row) {
+                                             StateAt state, const float o[3], const float d[3],
+                                             const float inv_d[3], float omax, int64_t row) {
     float C[3] = {0.f, 0.f, 0.f}, Cd[3] = {0.f, 0.f, 0.f}, F[4] = {0.f, 0.f, 0.f, 0.f}, T = 1.f;
     int nsamp = 0;
     for (int k = 0; k < n_blk; k++) {
         RayState sb = {{0.f, 0.f, 0.f}, {0.f, 0.f, 0.f, 0.f}, 1.f, 0, false};
         march_block<DT>(rec_at(k), o, d, inv_d, omax, a.ert_eps > 0.f ? a.ert_eps / T : 0.f, sb, a.err);
+        if (float *e = state(k)) {
+            const bool any = sb.nsamp > 0;
+            float4 *e4 = reinterpret_cast<float4 *>(e);
+            e4[0] = any ? make_float4(sb.Cd[0], sb.Cd[1], sb.Cd[2], sb.F[0]) : make_float4(0.f, 0.f, 0.f, 0.f);
+            e4[1] = any ? make_float4(sb.F[1], sb.F[2], sb.F[3], T) : make_float4(0.f, 0.f, 0.f, -1.f);
+        }
         if (sb.nsamp == 0) continue;
         float phi[3];
         block_mlp(mlp_at(k), a.n_freq, sb.Cd, sb.F, d, phi);
@@ -124,7 +131,8 @@ __device__ __forceinline__ void march_blocks_blend(const MarchArgs &a, const Vie
                                                    float omax, int64_t row) {
     blend_blocks<DT>(
         a, v.ids_count, [&](int k) -> const BlockRec & { return recs[k]; },
-        [&](int k) { return a.block_mlps[v.ids_begin + k]; }, o, d, inv_d, omax, row);
+        [&](int k) { return a.block_mlps[v.ids_begin + k]; }, [](int) -> float * { return nullptr; }, o, d, inv_d,
+        omax, row);
 }
 
 // One ray per thread of the tile: march the view's near-to-far block list
@@ -251,33 +259,22 @@ __device__ __forceinline__ void blend_blocks_warp(WarpScratch &ws, const MarchAr
     write_outputs_warp(a, row, CF, T, nsamp, C);
 }
 
-// A camera's rays given as a ray batch: three quarters of them enter where the
-// next ray enters, in its direction (32 consecutive rays can have 31 such).
-__device__ __forceinline__ bool rays_alike(const MarchArgs &a) {
-    return a.ray_alike && 4 * (int64_t)__ldg(a.ray_alike) >= 3 * a.n_rays;
-}
-
-// The ray form for such rays, one ray per thread in the given order: the rays
-// of a warp are neighbouring pixels, and their gathers share lines as the view
-// marcher's do (16 blocks of 128^3 FP16, the 921600 rays of a 720p camera: 9.2
-// ms, one ray per warp 13.4 ms).
+// The ray form, one ray per thread, where that is the faster one (ray_form in
+// cow_api.cu): the gathers of a camera's rays share lines in the given order, as
+// the view marcher's do.
 template <int DT, bool kBlockMlp>
 __global__ void __launch_bounds__(kThreads, kMinBlocks) k_march_rays_t(const __grid_constant__ MarchArgs a,
                                                                        const __grid_constant__ RayRecs rr) {
     __shared__ float s_mlp[kMlpParams + 1];
-    if (!rays_alike(a)) return;
+    bool given;
+    if (!thread_form(a, given)) return;
     if (!kBlockMlp) {
         load_mlp(a.mlp, s_mlp, (a.flags & 1u) != 0);
         __syncthreads();
     }
-    const int64_t r = (int64_t)blockIdx.x * kThreads + threadIdx.x;
-    if (r >= a.n_rays) return;
     float o[3], d[3];
-#pragma unroll
-    for (int c = 0; c < 3; c++) {
-        o[c] = __ldg(a.ray_o + 3 * r + c);
-        d[c] = __ldg(a.ray_d + 3 * r + c);
-    }
+    const int64_t r = load_ray(a, (int64_t)blockIdx.x * kThreads + threadIdx.x, given, o, d);
+    if (r < 0) return;
     int order[kMaxRayIds];
     const int n = sort_blocks_for_ray(rr, o, order);
     float inv_d[3], omax;
@@ -285,13 +282,26 @@ __global__ void __launch_bounds__(kThreads, kMinBlocks) k_march_rays_t(const __g
     if (kBlockMlp) {
         blend_blocks<DT>(
             a, n, [&](int k) -> const BlockRec & { return rr.r[order[k]]; },
-            [&](int k) { return a.block_mlp_base + (int64_t)rr.id[order[k]] * a.block_mlp_stride; }, o, d, inv_d, omax,
-            r);
+            [&](int k) { return a.block_mlp_base + (int64_t)rr.id[order[k]] * a.block_mlp_stride; },
+            [&](int k) -> float * {
+                return a.out_block_state ? a.out_block_state + 8 * (r * n + order[k]) : nullptr;
+            },
+            o, d, inv_d, omax, r);
         return;
     }
     RayState s = {{0.f, 0.f, 0.f}, {0.f, 0.f, 0.f, 0.f}, 1.f, 0, false};
-    for (int k = 0; k < n && !s.done; k++)
-        march_block<DT>(rr.r[order[k]], o, d, inv_d, omax, a.ert_eps, s, a.err);
+    if (a.out_block_T) {  // no early termination (k_march_rays)
+        float *bt = a.out_block_T + r * n;
+        for (int k = 0; k < n; k++) {
+            DepthSum tau;
+            const int n0 = s.nsamp;
+            march_block<DT>(rr.r[order[k]], o, d, inv_d, omax, a.ert_eps, s, a.err, &tau);
+            bt[order[k]] = s.nsamp > n0 ? tau.transmittance() : -1.f;
+        }
+    } else {
+        for (int k = 0; k < n && !s.done; k++)
+            march_block<DT>(rr.r[order[k]], o, d, inv_d, omax, a.ert_eps, s, a.err);
+    }
     write_outputs(a, r, s, d, s_mlp);
 }
 
@@ -300,7 +310,7 @@ __global__ void __launch_bounds__(kThreads, COW_RAYS_MIN_BLOCKS) k_march_rays(co
                                                                           const __grid_constant__ RayRecs rr) {
     __shared__ float s_mlp[kMlpParams + 1];
     __shared__ WarpScratch s_ws[kThreads / 32];
-    if (rays_alike(a)) return;  // k_march_rays_t has them
+    if (rays_alike(a)) return;  // the thread form has them
     if (!kBlockMlp) {
         load_mlp(a.mlp, s_mlp, (a.flags & 1u) != 0);
         __syncthreads();
@@ -359,6 +369,7 @@ template <int DT>
 __global__ void __launch_bounds__(kThreads, COW_RAYS_MIN_BLOCKS) k_march_partials(const __grid_constant__ MarchArgs a,
                                                                               const __grid_constant__ RayRecs rr) {
     __shared__ WarpScratch s_ws[kThreads / 32];
+    if (rays_alike(a)) return;
     WarpScratch &ws = s_ws[threadIdx.x >> 5];
     const int lane = threadIdx.x & 31;
     float o[3], d[3], inv_d[3], omax;
@@ -376,14 +387,24 @@ __global__ void __launch_bounds__(kThreads, COW_RAYS_MIN_BLOCKS) k_march_partial
     });
 }
 
-// Frames of up to this many pixels are marched one ray per warp: one ray per
-// thread then has every ray on the chip at once (152 SMs x 512 threads) and
-// takes as long as its longest ray.  Measured (us, thread / warp form): M = 1
-// block of 64^3 FP32, 128x128 357 / 98, 320x240 389 / 337, 400x300 488 / 525;
-// 4x4 blocks of 128^3 BF16, 96x54 2585 / 125, 320x240 2223 / 1382, 400x300
-// 2286 / 2113, 480x360 2662 / 2996; three-level city BF16, 96x54 2985 / 83,
-// 320x240 1885 / 666.
-constexpr int64_t kChipRays = 152 * kMinBlocks * kThreads;
+// The same, one ray per thread.
+template <int DT>
+__global__ void __launch_bounds__(kThreads, kMinBlocks) k_march_partials_t(const __grid_constant__ MarchArgs a,
+                                                                           const __grid_constant__ RayRecs rr) {
+    bool given;
+    if (!thread_form(a, given)) return;
+    float o[3], d[3], inv_d[3], omax;
+    const int64_t r = load_ray(a, (int64_t)blockIdx.x * kThreads + threadIdx.x, given, o, d);
+    if (r < 0) return;
+    ray_setup(d, o, inv_d, omax);
+    for (int k = 0; k < rr.n; k++) {
+        RayState s = {{0.f, 0.f, 0.f}, {0.f, 0.f, 0.f, 0.f}, 1.f, 0, false};
+        march_block<DT>(rr.r[k], o, d, inv_d, omax, 0.f, s, a.err);
+        float4 *pp = reinterpret_cast<float4 *>(a.out_partials + 8 * (r * rr.n + k));
+        pp[0] = make_float4(s.Cd[0], s.Cd[1], s.Cd[2], s.F[0]);
+        pp[1] = make_float4(s.F[1], s.F[2], s.F[3], s.T);
+    }
+}
 
 // One ray per warp over a view's near-to-far block list.
 template <int DT, bool kBlockMlp>
@@ -491,7 +512,7 @@ cudaError_t launch_views_dt(const MarchArgs &a, int n_tiles, int schedule, cudaS
     }
     const bool in_params = schedule == kSchedThreadConst;
     if (in_params && !pr) return cudaErrorInvalidValue;
-    if (in_params && a.n_rays <= kChipRays) {
+    if (in_params && a.form == kFormWarp) {
         if (block_mlp) k_march_views_cw<DT, true><<<n_tiles * 32, kThreads, 0, st>>>(a, *pr);
         else k_march_views_cw<DT, false><<<n_tiles * 32, kThreads, 0, st>>>(a, *pr);
         return cudaGetLastError();
@@ -500,23 +521,28 @@ cudaError_t launch_views_dt(const MarchArgs &a, int n_tiles, int schedule, cudaS
                      : launch_thread<DT, false>(a, n_tiles, in_params, st, pr);
 }
 
+// kFormWarp with a count of alike rays: both forms are launched, and the count
+// decides on the device which of them returns at once.
 template <int DT>
 cudaError_t launch_rays_dt(const MarchArgs &a, const RayRecs &rr, cudaStream_t st) {
-    const int64_t nb = (a.n_rays + kThreads / 32 - 1) / (kThreads / 32);
-    if (a.ray_alike) {  // decided on the device by the count of alike rays: the other of the two kernels returns at once
-        const unsigned nt = (unsigned)((a.n_rays + kThreads - 1) / kThreads);
+    const unsigned nw = (unsigned)((a.n_rays + kThreads / 32 - 1) / (kThreads / 32));
+    const unsigned nt = (unsigned)((a.n_rays + kThreads - 1) / kThreads);
+    if (a.form == kFormThread || a.ray_alike) {
         if (a.block_mlp_base) k_march_rays_t<DT, true><<<nt, kThreads, 0, st>>>(a, rr);
         else k_march_rays_t<DT, false><<<nt, kThreads, 0, st>>>(a, rr);
     }
-    if (a.block_mlp_base) k_march_rays<DT, true><<<(unsigned)nb, kThreads, 0, st>>>(a, rr);
-    else k_march_rays<DT, false><<<(unsigned)nb, kThreads, 0, st>>>(a, rr);
+    if (a.form == kFormThread) return cudaGetLastError();
+    if (a.block_mlp_base) k_march_rays<DT, true><<<nw, kThreads, 0, st>>>(a, rr);
+    else k_march_rays<DT, false><<<nw, kThreads, 0, st>>>(a, rr);
     return cudaGetLastError();
 }
 
 template <int DT>
 cudaError_t launch_partials_dt(const MarchArgs &a, const RayRecs &rr, cudaStream_t st) {
-    const int64_t nb = (a.n_rays + kThreads / 32 - 1) / (kThreads / 32);
-    k_march_partials<DT><<<(unsigned)nb, kThreads, 0, st>>>(a, rr);
+    const unsigned nw = (unsigned)((a.n_rays + kThreads / 32 - 1) / (kThreads / 32));
+    const unsigned nt = (unsigned)((a.n_rays + kThreads - 1) / kThreads);
+    if (a.form == kFormThread || a.ray_alike) k_march_partials_t<DT><<<nt, kThreads, 0, st>>>(a, rr);
+    if (a.form == kFormWarp) k_march_partials<DT><<<nw, kThreads, 0, st>>>(a, rr);
     return cudaGetLastError();
 }
 

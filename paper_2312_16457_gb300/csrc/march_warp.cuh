@@ -302,19 +302,39 @@ __device__ __forceinline__ void for_each_hit(int n, RecAt rec_at, const float o[
 }
 
 // Ray t in the call's order (a: the ray arrays and the order of a ray-batch
-// call): its index, or -1 beyond the last.
-__device__ __forceinline__ int64_t first_ray() { return (int64_t)blockIdx.x * (blockDim.x >> 5) + (threadIdx.x >> 5); }
-
+// call; given: the order is the given one): its index, or -1 beyond the last.
 template <class Args>
-__device__ __forceinline__ int64_t load_ray_warp(const Args &a, int64_t t, float o[3], float d[3]) {
+__device__ __forceinline__ int64_t load_ray(const Args &a, int64_t t, bool given, float o[3], float d[3]) {
     if (t >= a.n_rays) return -1;
-    const int64_t r = a.ray_perm ? (int64_t)__ldg(a.ray_perm + t) : t;
+    const int64_t r = a.ray_perm && !given ? (int64_t)__ldg(a.ray_perm + t) : t;
 #pragma unroll
     for (int c = 0; c < 3; c++) {
         o[c] = __ldg(a.ray_o + 3 * r + c);
         d[c] = __ldg(a.ray_d + 3 * r + c);
     }
     return r;
+}
+
+template <class Args>
+__device__ __forceinline__ int64_t load_ray_warp(const Args &a, int64_t t, float o[3], float d[3]) {
+    return load_ray(a, t, false, o, d);
+}
+
+// The warp's ray in the call's order.
+__device__ __forceinline__ int64_t first_ray() { return (int64_t)blockIdx.x * (blockDim.x >> 5) + (threadIdx.x >> 5); }
+
+// A camera's rays given as a ray batch: three quarters of them enter and leave
+// the blocks' box where the next ray does (32 consecutive rays can have 31 such).
+template <class Args>
+__device__ __forceinline__ bool rays_alike(const Args &a) {
+    return a.ray_alike && mostly_alike(__ldg(a.ray_alike), a.n_rays);
+}
+
+// Whether the thread form has the call, and whether in the given order.
+template <class Args>
+__device__ __forceinline__ bool thread_form(const Args &a, bool &given) {
+    given = rays_alike(a);
+    return given || a.form == kFormThread;
 }
 
 // deferred_mlp with lane j < 16 on hidden unit j (the same sums in the same

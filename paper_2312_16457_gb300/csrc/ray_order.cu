@@ -171,7 +171,7 @@ KeyGrid key_grid(const float lo[3], const float hi[3]) {
     return {make_float3(lo[0], lo[1], lo[2]), make_float3(hi[0], hi[1], hi[2]), axes, make_int3(nb[0], nb[1], nb[2])};
 }
 
-int key_blocks(int64_t n) { return (int)std::min<int64_t>((n + 255) / 256, 152 * 16); }
+int key_blocks(int64_t n) { return (int)std::min<int64_t>((n + 255) / 256, kSms * 16); }
 
 }  // namespace
 

@@ -105,3 +105,167 @@ def test_early_termination_in_front_of_nan_features(block_mlps):
             assert float((a - b).abs().max()) <= 1e-5 * float(a.abs().max())
     assert int(out[0][5].min()) > 8
     ctx.close()
+
+
+FORMS = ["fp32", "fp16", "bf16_fp8", "fp8 bricks", "fp8_bf16d bricks", "fp16 unbounded"]
+
+
+def _scene(opt):
+    if "unbounded" in opt:
+        return synth.workload_unbounded(R=21, P=67, width=37, height=29)[0]
+    return _city()
+
+
+def _rays(opt, sc, n):
+    o, d = synth.random_rays(n, 12, sc.box_lo, sc.box_hi)
+    if "unbounded" in opt:
+        o = torch.tensor([0.25, -0.4, 0.3]).expand(n, 3).contiguous()
+    return o.cuda(), d.cuda()
+
+
+def _marches(ctx, sc, o, d, mlp, ids):
+    """Every ray call that chooses a form: (calls, opacity gradients)."""
+    out = list(ctx.render_rays(o, d, ids, mlp, ert_eps=1e-2, nsamp=True))
+    out += list(ctx.render_rays(o, d, ids, None, ert_eps=1e-2, nsamp=True, block_mlps=True))
+    out += [*ctx.render_rays_block_t(o, d, ids, mlp)[:2], *ctx.render_rays_block_state(o, d, ids)]
+    out.append(ctx.render_partials(o, d, ids))
+    bt = ctx.render_rays_block_t(o, d, ids, mlp)[2]
+    grads = []
+    for T in (None, bt):
+        gg = [torch.zeros(b.grid.shape, device="cuda") for b in sc.blocks]
+        gp = [[torch.zeros(p.shape, device="cuda") for p in b.planes] for b in sc.blocks]
+        grads.append([ctx.opacity_loss(o, d, ids, 0.5, grads=(gg, gp), block_T=T), *gg, *sum(gp, [])])
+    return out, bt, grads
+
+
+@pytest.mark.parametrize("form", FORMS)
+def test_ray_calls_do_not_depend_on_the_form(form):
+    """Every march of a ray batch in both forms: outputs, sample counts and
+    per-block states bit for bit; what is summed in another order (the optical
+    depth of a block, the opacity loss and its gradient) to FP32 rounding."""
+    storage, *opt = form.split()
+    sc = _scene(opt)
+    o, d = _rays(opt, sc, 1003)
+    mlp = torch.from_numpy(synth.mlp_weights(9)).cuda()
+    ctx = cow.Context(sc, storage, bricks="bricks" in opt)
+    ctx.set_block_mlps(synth.block_mlp_weights(3, 4, 2), 2)
+    res = []
+    for f in ("thread", "warp"):
+        ctx.set_test_hooks(form=f)
+        res.append(_marches(ctx, sc, o, d, mlp, IDS))
+        assert ctx.last_form() == f
+    ctx.set_test_hooks()
+    ctx.sync_check()
+    (a, bt_a, ga), (b, bt_b, gb) = res
+    for x, y in zip(a, b):
+        assert torch.equal(x, y)
+    assert torch.equal(bt_a < 0, bt_b < 0) and int((bt_a >= 0).sum()) > 500
+    # exp(-tau): tau of up to ~300 samples, whose 32 lane sums carry some 10 roundings
+    # of a partial sum each: 2^-24 (10 + 5) tau exp(-tau) at most, tau exp(-tau) <= 0.37
+    assert float((bt_a - bt_b).abs().max()) <= 5e-7
+    for x, y in zip(ga, gb):
+        for u, v in zip(x, y):
+            assert float((u - v).abs().max()) <= 1e-4 * float(v.abs().max()) + 1e-12
+    ctx.close()
+
+
+@pytest.mark.parametrize("order", ["coherent", "given"])
+@pytest.mark.parametrize("form", ["fp32", "bf16_fp8", "fp8 bricks", "fp16 unbounded"])
+def test_camera_rays_take_the_thread_form(form, order):
+    """A camera's 2^17 rays and more (not a whole number of CTAs) take the thread
+    form in every march, the same rays shuffled the warp form, with the same
+    results, also where only seven tenths of the rays are the camera's."""
+    storage, *opt = form.split()
+    sc = _scene(opt)
+    mlp = torch.from_numpy(synth.mlp_weights(9)).cuda()
+    ctx = cow.Context(sc, storage, bricks="bricks" in opt)
+    ctx.set_block_mlps(synth.block_mlp_weights(3, 4, 2), 2)
+    ctx.set_ray_order(order)
+    o, d = _camera_rays(500, 301)
+    if "unbounded" in opt:
+        o = o + torch.tensor([2.6, 3.1, -1.6], device="cuda")
+    n = o.shape[0]
+    perm = torch.randperm(n, generator=torch.Generator().manual_seed(1)).cuda()
+    mixed = torch.cat([torch.arange(n * 7 // 10, device="cuda"), perm[perm >= n * 7 // 10]])
+    calls = [lambda o, d: ctx.render_rays(o, d, IDS, mlp, ert_eps=1e-3, nsamp=True),
+             lambda o, d: ctx.render_rays(o, d, IDS, None, ert_eps=1e-3, nsamp=True, block_mlps=True),
+             lambda o, d: ctx.render_rays_block_t(o, d, IDS, mlp)[:2],
+             lambda o, d: ctx.render_rays_block_state(o, d, IDS),
+             lambda o, d: [ctx.render_partials(o, d, IDS)]]
+    for call in calls:
+        want = call(o, d)
+        assert ctx.last_form() == "thread"
+        for p in (perm, mixed):
+            got = call(o[p], d[p])
+            assert ctx.last_form() == "warp"
+            for x, y in zip(got, want):
+                assert torch.equal(x, y[p])
+    loss = ctx.opacity_loss(o, d, IDS)
+    assert ctx.last_form() == "thread"
+    again = ctx.opacity_loss(o[perm], d[perm], IDS)
+    assert ctx.last_form() == "warp"
+    assert abs(float(loss) - float(again)) <= 1e-5 * float(loss)
+    ctx.sync_check()
+    ctx.close()
+
+
+@pytest.mark.parametrize("form", ["fp32", "fp16 unbounded"])
+def test_gradients_of_camera_rays_with_the_thread_forms_totals(form):
+    """The backward of a camera's rays takes its totals from the thread form and
+    marches one ray per warp: the same gradients as with the warp form's totals,
+    and as the sum in 64 bits over 64 calls."""
+    storage, *opt = form.split()
+    sc = _scene(opt)
+    mlp = torch.from_numpy(synth.mlp_weights(9)).cuda()
+    ctx = cow.Context(sc, storage)
+    o, d = _camera_rays(500, 301)
+    if "unbounded" in opt:
+        o = o + torch.tensor([2.6, 3.1, -1.6], device="cuda")
+    n = o.shape[0]
+    g = torch.randn((n, 3), generator=torch.Generator().manual_seed(2)).cuda() / n
+
+    def grad(part, aux):
+        gg = [torch.zeros(b.grid.shape, device="cuda") for b in sc.blocks]
+        gp = [[torch.zeros(p.shape, device="cuda") for p in b.planes] for b in sc.blocks]
+        gm = torch.zeros(499, device="cuda")
+        ctx.render_backward(o[part], d[part], IDS, mlp, aux[part], g[part], gg, gp, gm)
+        return [gm, *gg, *sum(gp, [])]
+
+    auxs = []
+    for f in ("thread", "warp"):
+        ctx.set_test_hooks(form=f)
+        auxs.append(ctx.render_rays(o, d, IDS, mlp)[1])
+    ctx.set_test_hooks()
+    assert torch.equal(*auxs)
+    got, want = grad(slice(None), auxs[0]), None
+    for k in range(64):
+        part = [x.double() for x in grad(slice(k * n // 64, (k + 1) * n // 64), auxs[0])]
+        want = part if want is None else [a + b for a, b in zip(want, part)]
+    ctx.sync_check()
+    for a, b in zip(got, want):
+        assert float((a.double() - b).abs().max()) <= 1e-4 * float(b.abs().max())
+    ctx.close()
+
+
+@pytest.mark.parametrize("ert", [0.0, 1e-2])
+@pytest.mark.parametrize("form", FORMS + ["bf16 block_mlps"])
+def test_views_do_not_depend_on_the_form(form, ert):
+    storage, *opt = form.split()
+    sc = _scene(opt)
+    ctx = cow.Context(sc, storage, bricks="bricks" in opt)
+    bm = "block_mlps" in opt
+    if bm:
+        ctx.set_block_mlps(synth.block_mlp_weights(3, 4, 3), 3)
+    cam = synth.camera((-0.6, -0.5, 0.6) if "unbounded" in opt else (-2.6, -3.1, 2.0), (0.9, 0.8, -0.5), 37, 29, 60.0)
+    ids = ctx.sort_blocks(cam, IDS)
+    res = []
+    for f in ("thread", "warp"):
+        ctx.set_test_hooks(form=f)
+        res.append(ctx.render([cam], [ids], synth.mlp_weights(9), ert_eps=ert, nsamp=True, block_mlps=bm))
+        assert ctx.last_form() == f
+    ctx.set_test_hooks()
+    ctx.sync_check()
+    for x, y in zip(*res):
+        assert torch.equal(x, y)
+    assert int(res[0][2].max()) > 64
+    ctx.close()
