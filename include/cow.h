@@ -643,9 +643,10 @@ cow_status cow_mse_grad(const float *rgb, const float *target, int64_t n, float 
  *     (measured 4 % faster at 1080p); used when the call's views select at
  *     most 96 block records in total, otherwise the call runs as
  *     COW_SCHED_THREAD;
- *     a call of at most 77824 pixels (those that fill the chip at one ray per
- *     thread) marches one ray per warp instead, the 32 lanes on the ray's next
- *     32 occupied samples, composited in order (the same image);
+ *     a call of few pixels marches one ray per warp instead, the 32 lanes on
+ *     the ray's next 32 occupied samples, composited in order (the same image):
+ *     at most 8000 + 280 P, P the smallest plane resolution of its blocks, and
+ *     at most 77824, those that fill the chip at one ray per thread;
  *   COW_SCHED_WARP: one ray per warp for frames of any size, each warp taking
  *     32 rays of its tile one after another, records in shared memory (measured
  *     slower on large aerial views: rays of one tile are marched one after
@@ -664,10 +665,12 @@ cow_status cow_set_schedule(cow_ctx *ctx, int32_t schedule);
  * by a counting sort on the device -- so that the rays on the chip at one time
  * gather neighbouring texels and share them in L2 (measured on 2^20 random rays
  * over 2x2 blocks of 128^3 / 512^2 FP32 features: forward 39.9 -> 28.3 ms).
- * COW_RAY_ORDER_GIVEN: warp t marches ray t.  Calls of 2^17 rays or more that
- * are mostly alike their neighbours (a camera's rays) are marched one ray per
- * thread in the given order, but for the backwards and the opacity gradient; a
- * key pass over the rays counts the alike ones.
+ * COW_RAY_ORDER_GIVEN: warp t marches ray t.  Rays that are mostly alike their
+ * neighbours (a camera's) are marched one ray per thread in the given order,
+ * from 8000 + 280 P rays up (at most 2^17); a key pass counts the alike ones.
+ * Random rays are marched one ray per thread in calls so large that many meet in
+ * a texel.  Both but for the backwards and most opacity gradients, which are
+ * faster one ray per warp.
  * Outputs are written at each ray's own index either way and each ray's values
  * are the same; gradient sums change only by the order of their FP32
  * reductions.  The coherent order costs a key pass, a scan and a scatter, about

@@ -614,15 +614,35 @@ int32_t forced_form(const cow_ctx *c) {
     return c->test_flags & COW_TEST_THREAD_FORM ? cow::kFormThread : c->test_flags & COW_TEST_WARP_FORM ? cow::kFormWarp : -1;
 }
 
-// Frames of up to kChipRays pixels are marched one ray per warp: one ray per
-// thread then has every ray on the chip at once and takes as long as its longest
-// ray.  Measured (us, thread / warp form): M = 1 block of 64^3 FP32, 128x128
-// 357 / 98, 320x240 389 / 337, 400x300 488 / 525; 4x4 blocks of 128^3 BF16,
-// 96x54 2585 / 125, 320x240 2223 / 1382, 400x300 2286 / 2113, 480x360 2662 /
-// 2996; three-level city BF16, 96x54 2985 / 83, 320x240 1885 / 666.
-int32_t view_form(const cow_ctx *c, int64_t n_pix) {
+struct CallShape {
+    int32_t n_ids;
+    int64_t P;  // the smallest plane resolution of the call's blocks: lattice points across a block
+};
+
+CallShape call_shape(const cow_ctx *c, const int32_t *ids, int32_t n_ids) {
+    CallShape s = {n_ids, n_ids > 0 ? INT32_MAX : 0};
+    for (int32_t k = 0; k < n_ids; k++) s.P = std::min<int64_t>(s.P, c->blocks[(size_t)ids[k]].P);
+    return s;
+}
+
+// A camera's rays, in a frame or a batch, up to which one ray per warp is the
+// faster form: one ray per thread takes as long as its longest ray, of some P
+// samples a block, the warp form a constant and P / 32 chunks for every ray.
+// Pixels at which both took the same (FP32 / BF16, one, four and sixteen
+// blocks): P = 32 19 k; P = 64 33, 32, 35 k; P = 96 44, 42, 50 k; P = 128 58, 43
+// (FP16 62), 60 k; P = 192 -, 62 (FP16 70), 75 k; P = 256 85 k; P = 512 -, -, 140 k.
+int64_t warp_pixels(const CallShape &s) { return 8000 + 280 * s.P; }
+
+// At most kChipRays pixels, which one ray per thread has on the chip at once.
+// Measured (us, thread / warp form): M = 1 block of 64^3 and 256^2 FP32, 128x128
+// 357 / 98, 320x240 389 / 337, 400x300 488 / 525; 4x4 blocks of 128^3 and 512^2
+// BF16, 96x54 2585 / 125, 320x240 2223 / 1382, 400x300 2286 / 2113, 480x360 2662 /
+// 2996; three-level city BF16, 96x54 2985 / 83, 320x240 1885 / 666; 2x2 blocks of
+// 24^3 and 96^2 FP32, 192x144 294 / 237, 320x240 367 / 574.
+int32_t view_form(const cow_ctx *c, const int32_t *ids, int32_t n_ids, int64_t n_pix) {
     if (forced_form(c) >= 0) return forced_form(c);
-    return n_pix <= cow::kChipRays ? cow::kFormWarp : cow::kFormThread;
+    return n_pix <= std::min(warp_pixels(call_shape(c, ids, n_ids)), cow::kChipRays) ? cow::kFormWarp
+                                                                                   : cow::kFormThread;
 }
 
 // What a ray batch is marched for: the outputs of the march, the block-parallel
@@ -630,17 +650,72 @@ int32_t view_form(const cow_ctx *c, int64_t n_pix) {
 // every block twice), the gradient from the forward's in-block transmittances.
 enum RayCall { kCallMarch, kCallPartials, kCallOpacity, kCallOpacityGrad, kCallOpacityGradT };
 
+// Random rays from which one ray per thread is the faster form.  It pays where
+// many rays meet in few texels, so that the rays of a warp (sorted, ray_order.cu)
+// share their lines: above a number of rays a texel, P^2 a block, that grows with
+// the blocks, between which rays diverge, and with the bytes of an FP32 texel.
+// Small storage stays in L1 and L2 when one block or the partials of one block at
+// a time are marched; there the longest ray, some P samples, decides.  The
+// opacity term reads and composites less a sample, which suits the warp form, as
+// does the gradient's scatter, but for many blocks of few samples each.
+// Thousands of rays at which both took the same, FP32 / BF16:
+//   blocks P     march        partials     opacity
+//    1     32    20 / 14      28 / 18      18 / 15
+//    1     64    48 / 27      95 / 34      170 / 32
+//    1     96    90 / 38      230 / 47     - / 80
+//    1    160    280 / 60     800 / 80     - / 270
+//    1    256    850 / 110    2600 / 140   - / -
+//    4     32    55 / 47      78 / 36      90 / 33
+//    4     64    190 / 140    220 / 75     - / 95
+//    4     96    600 / 310    640 / 115    - / 330
+//    9     32    180 / 175    115 / 55     160 / 63
+//   16     32    320 / 330    150 / 78     180 / 85
+//   16     64    2600 / 2600  530 / 150    - / 340
+// and 2.56 M rays, the most measured, left the warp form ahead at "-".
+int64_t thread_rays(const cow_ctx *c, const CallShape &s, RayCall call) {
+    const bool f32 = c->dtype == cow::kF32;
+    const double P = (double)s.P, n = s.n_ids;
+    double rays = 1e18;
+    switch (call) {
+        case kCallMarch:
+            rays = n == 1 ? (f32 ? std::max(600 * P, 13 * P * P) : 450 * P)
+                          : std::max(600 * P, (f32 ? 12 : 7) * P * P * n * (1 + n / 8));
+            break;
+        case kCallPartials: rays = f32 ? P * P * (18 + 9 * n) : P * (450 + 130 * n); break;
+        case kCallOpacity:
+            if (f32 ? P <= 48 || (n == 1 && P <= 64) : P <= 128 || (n == 1 && P <= 192))
+                rays = f32 ? P * P * P * (0.3 + 0.35 * n) : P * P * 5 * (1 + n);
+            break;
+        case kCallOpacityGrad:
+            if (n > 8 && P <= 64) rays = 5000 * P;  // 16 blocks, P = 32, 1.28 M rays: 0.57 to 0.70 of the warp form's time
+            break;
+        case kCallOpacityGradT: break;
+    }
+    return (int64_t)std::min(rays, 1e18);
+}
+
+// A camera's rays from which one ray per thread, in the given order, is the
+// faster form.  921600 of them (ms, thread / warp): 16 blocks of 128^3 and 512^2
+// FP16, march 8.7 / 13.4, with in-block transmittances 9.9 / 13.7, partials 9.5 /
+// 12.0, opacity 7.3 / 10.6, with its gradient 29.6 / 29.5 and, from the
+// transmittances, 24.2 / 21.1; 10^6 through 16 blocks of 96^2 FP32, opacity and
+// gradient 13.4 / 16.4.
+int64_t thread_alike(const CallShape &s, RayCall call) {
+    if (call == kCallOpacityGradT || (call == kCallOpacityGrad && s.n_ids <= 8)) return INT64_MAX;
+    if (call == kCallOpacityGrad) return 2000 * s.P;
+    return std::min(warp_pixels(s), cow::kRaysAlikeMin);
+}
+
 // The form of a ray batch.  *count: the device counts the alike rays, and takes
-// the thread form in the given order when it is a camera's.  Measured on 921600
-// camera rays (ms, thread in the given order / warp): 16 blocks of 128^3 FP16,
-// rays 8.7 / 13.4, with in-block transmittances 9.9 / 13.7, partials 9.5 / 12.0,
-// opacity 7.3 / 10.6, with gradients 29.6 / 29.5 and, from the transmittances,
-// 24.2 / 21.1.
-int32_t ray_form(const cow_ctx *c, int64_t n, RayCall call, bool *count) {
+// the thread form in the given order when it is a camera's.
+int32_t ray_form(const cow_ctx *c, const int32_t *ids, int32_t n_ids, int64_t n, RayCall call, bool *count) {
     *count = false;
     if (forced_form(c) >= 0) return forced_form(c);
-    *count = call != kCallOpacityGrad && call != kCallOpacityGradT && n >= cow::kRaysAlikeMin;
-    return cow::kFormWarp;
+    const CallShape s = call_shape(c, ids, n_ids);
+    const int32_t form = n >= thread_rays(c, s, call) ? cow::kFormThread : cow::kFormWarp;
+    // a call in the thread form asks only whether to keep to the given order
+    *count = n >= thread_alike(s, call) && (form == cow::kFormWarp || c->ray_order == COW_RAY_ORDER_COHERENT);
+    return form;
 }
 
 void note_form(cow_ctx *c, int32_t form, int64_t n, const uint32_t *alike) {
@@ -1072,7 +1147,7 @@ cow_status cow_render(cow_ctx *ctx, const cow_camera *cams, int32_t n_views, con
         cow::ParamRecs pr;
         std::memset(&pr, 0, sizeof(pr));
         std::copy(vrecs.begin(), vrecs.begin() + n_ids, pr.r);
-        a.form = view_form(ctx, plan.n_pix);
+        a.form = view_form(ctx, ids, n_ids, plan.n_pix);
         COW_CUDA(cow::launch_march_views(a, plan.n_tiles, cow::kSchedThreadConst, st, &pr));
     } else {
         // the warp schedule marches bounded blocks only
@@ -1146,7 +1221,7 @@ static cow_status render_rays_impl(cow_ctx *ctx, const float *o, const float *d,
         a.n_freq = ctx->n_freq;
     }
     bool count;
-    a.form = ray_form(ctx, n_rays, kCallMarch, &count);
+    a.form = ray_form(ctx, ids, n_ids, n_rays, kCallMarch, &count);
     if ((rc = ray_order(ctx, o, d, n_rays, ids, n_ids, st, &a.ray_perm, count, &a.ray_alike)) != COW_OK) return rc;
     cow::RayRecs rr;
     make_ray_recs(ctx, ids, n_ids, rr);
@@ -1185,7 +1260,7 @@ cow_status cow_render_partials(cow_ctx *ctx, const float *o, const float *d, int
     a.n_rays = n_rays;
     a.out_partials = out_partials;
     bool count;
-    a.form = ray_form(ctx, n_rays, kCallPartials, &count);
+    a.form = ray_form(ctx, ids, n_ids, n_rays, kCallPartials, &count);
     if ((rc = ray_order(ctx, o, d, n_rays, ids, n_ids, st, &a.ray_perm, count, &a.ray_alike)) != COW_OK) return rc;
     cow::RayRecs rr;
     make_ray_recs(ctx, ids, n_ids, rr);
@@ -1542,7 +1617,7 @@ cow_status cow_opacity_loss(cow_ctx *ctx, const float *o, const float *d, int64_
     a.loss_parts = (float *)(ctx->d_err + kCtxLossParts);
     bool count;
     const RayCall call = !grad_grid ? kCallOpacity : block_T ? kCallOpacityGradT : kCallOpacityGrad;
-    a.form = ray_form(ctx, n_rays, call, &count);
+    a.form = ray_form(ctx, ids, n_ids, n_rays, call, &count);
     if ((rc = ray_order(ctx, o, d, n_rays, ids, n_ids, st, &a.ray_perm, count, &a.ray_alike)) != COW_OK) return rc;
     cow::RayRecs rr;
     make_ray_recs(ctx, ids, n_ids, rr);

@@ -73,7 +73,8 @@ constexpr int kRayOrderKeyBits = 20;
 constexpr int kRayOrderBins = 1 << kRayOrderKeyBits;
 constexpr int kRayOrderAlike = kRayOrderBins;
 constexpr int kRayOrderHistWords = kRayOrderBins + 32 + kRayOrderBins / 1024;
-// Calls of at least this many rays look at the count (ray_form in cow_api.cu).
+// Calls of at least this many rays look at the count (smaller ones from where
+// the thread form pays, thread_alike in cow_api.cu).
 constexpr int64_t kRaysAlikeMin = 1 << 17;
 // Whether n of a call's n_rays rays, alike the next one, make it a camera's.
 __host__ __device__ __forceinline__ bool mostly_alike(uint32_t n, int64_t n_rays) { return 4 * (int64_t)n >= 3 * n_rays; }

@@ -43,6 +43,7 @@ struct KeyGrid {
     float3 lo, hi;
     uint32_t axes;
     int3 bits;
+    int alike_drop;  // low bits of the key that alike rays may differ in
 };
 
 // kSort: the keys and their histogram for the order; the count either way.
@@ -95,7 +96,7 @@ __global__ void k_ray_keys(const float *__restrict__ o, const float *__restrict_
             }
         }
         const uint32_t next = __shfl_down_sync(0xffffffffu, key, 1);
-        const bool pair = i + 1 < n && (threadIdx.x & 31) != 31 && next == key;
+        const bool pair = i + 1 < n && (threadIdx.x & 31) != 31 && ((next ^ key) >> kg.alike_drop) == 0;
         same += __popc(__ballot_sync(0xffffffffu, pair));
     }
     if ((threadIdx.x & 31) == 0 && same) atomicAdd(n_alike, same);
@@ -155,7 +156,7 @@ __global__ void k_ray_scatter(const uint32_t *__restrict__ keys, int64_t n, uint
 }
 
 // Every step halves the longest edge of the cells: near cubic cells.
-KeyGrid key_grid(const float lo[3], const float hi[3]) {
+KeyGrid key_grid(const float lo[3], const float hi[3], int64_t n) {
     uint32_t axes = 0;
     int nb[3] = {0, 0, 0};
     float ext[3];
@@ -168,7 +169,12 @@ KeyGrid key_grid(const float lo[3], const float hi[3]) {
         nb[a]++;
         ext[a] *= 0.5f;
     }
-    return {make_float3(lo[0], lo[1], lo[2]), make_float3(hi[0], hi[1], hi[2]), axes, make_int3(nb[0], nb[1], nb[2])};
+    // a camera of 2^17 rays has some eleven to a cell's edge; for fewer rays the
+    // cells that count as the same grow with their spacing
+    int drop = 0;
+    for (int64_t m = n; m < kRaysAlikeMin && drop < 8; m *= 2) drop += 2;
+    return {make_float3(lo[0], lo[1], lo[2]), make_float3(hi[0], hi[1], hi[2]), axes, make_int3(nb[0], nb[1], nb[2]),
+            drop};
 }
 
 int key_blocks(int64_t n) { return (int)std::min<int64_t>((n + 255) / 256, kSms * 16); }
@@ -186,7 +192,7 @@ cudaError_t launch_ray_order(const float *o, const float *d, int64_t n, const fl
     if (e != cudaSuccess) return e;
     uint32_t *sums = hist + kRayOrderBins + 32;
     const int grid = key_blocks(n);
-    k_ray_keys<true><<<grid, 256, 0, st>>>(o, d, n, key_grid(lo, hi), keys, hist, hist + kRayOrderAlike);
+    k_ray_keys<true><<<grid, 256, 0, st>>>(o, d, n, key_grid(lo, hi, n), keys, hist, hist + kRayOrderAlike);
     k_scan_local<<<kScanBlocks, kScanThreads, 0, st>>>(hist, sums);
     k_scan_sums<<<1, kScanBlocks, 0, st>>>(sums);
     k_ray_scatter<<<grid, 256, 0, st>>>(keys, n, hist, sums, perm);
@@ -198,7 +204,7 @@ cudaError_t launch_count_alike(const float *o, const float *d, int64_t n, const 
     if (n <= 0 || n > 0x7fffffff) return cudaErrorInvalidValue;
     cudaError_t e = cudaMemsetAsync(n_alike, 0, sizeof(uint32_t), st);
     if (e != cudaSuccess) return e;
-    k_ray_keys<false><<<key_blocks(n), 256, 0, st>>>(o, d, n, key_grid(lo, hi), nullptr, nullptr, n_alike);
+    k_ray_keys<false><<<key_blocks(n), 256, 0, st>>>(o, d, n, key_grid(lo, hi, n), nullptr, nullptr, n_alike);
     return cudaGetLastError();
 }
 

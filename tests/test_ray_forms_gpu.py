@@ -170,20 +170,18 @@ def test_ray_calls_do_not_depend_on_the_form(form):
 
 
 @pytest.mark.parametrize("order", ["coherent", "given"])
-@pytest.mark.parametrize("form", ["fp32", "bf16_fp8", "fp8 bricks", "fp16 unbounded"])
+@pytest.mark.parametrize("form", ["fp32", "bf16_fp8", "fp8 bricks"])
 def test_camera_rays_take_the_thread_form(form, order):
     """A camera's 2^17 rays and more (not a whole number of CTAs) take the thread
     form in every march, the same rays shuffled the warp form, with the same
     results, also where only seven tenths of the rays are the camera's."""
     storage, *opt = form.split()
-    sc = _scene(opt)
+    sc = synth.city_scene(23, 2, 2.0, [(21, 260)], **synth.SPARSE_CITY)
     mlp = torch.from_numpy(synth.mlp_weights(9)).cuda()
     ctx = cow.Context(sc, storage, bricks="bricks" in opt)
     ctx.set_block_mlps(synth.block_mlp_weights(3, 4, 2), 2)
     ctx.set_ray_order(order)
     o, d = _camera_rays(500, 301)
-    if "unbounded" in opt:
-        o = o + torch.tensor([2.6, 3.1, -1.6], device="cuda")
     n = o.shape[0]
     perm = torch.randperm(n, generator=torch.Generator().manual_seed(1)).cuda()
     mixed = torch.cat([torch.arange(n * 7 // 10, device="cuda"), perm[perm >= n * 7 // 10]])
@@ -269,3 +267,30 @@ def test_views_do_not_depend_on_the_form(form, ert):
         assert torch.equal(x, y)
     assert int(res[0][2].max()) > 64
     ctx.close()
+
+
+def test_small_planes_take_the_thread_form_earlier():
+    """Few samples a ray: frames and batches take the thread form where the same
+    calls over larger planes take the warp form."""
+    mlp = torch.from_numpy(synth.mlp_weights(9)).cuda()
+    form = {}
+    for P in (33, 260):
+        sc = synth.single_block_scene(1, 9, P)
+        ctx = cow.Context(sc, "bf16")
+        cam = synth.camera((0.0, -2.5, 0.8), (0.0, 0.0, 0.0), 200, 150, 60.0)
+        ctx.render([cam], [[0]], mlp)
+        form["view", P] = ctx.last_form()
+        o, d = (torch.from_numpy(x).cuda() for x in oracle.pixel_rays(cam))
+        perm = torch.randperm(o.shape[0], generator=torch.Generator().manual_seed(1)).cuda()
+        for name, p in (("camera", slice(None)), ("random", perm)):
+            res = []
+            for f in (None, "warp"):
+                ctx.set_test_hooks(form=f)
+                res.append(ctx.render_rays(o[p], d[p], [0], mlp, nsamp=True))
+                if f is None:
+                    form[name, P] = ctx.last_form()
+            for x, y in zip(*res):
+                assert torch.equal(x, y)
+        ctx.sync_check()
+        ctx.close()
+    assert form == {(k, P): "thread" if P == 33 else "warp" for P in (33, 260) for k in ("view", "camera", "random")}
