@@ -646,7 +646,8 @@ cow_status cow_mse_grad(const float *rgb, const float *target, int64_t n, float 
  *     a call of few pixels marches one ray per warp instead, the 32 lanes on
  *     the ray's next 32 occupied samples, composited in order (the same image):
  *     at most 8000 + 280 P, P the smallest plane resolution of its blocks, and
- *     at most 77824, those that fill the chip at one ray per thread;
+ *     at most 77824, those that fill the chip at one ray per thread; with
+ *     unbounded blocks at most 11000 + 45 P and 20000;
  *   COW_SCHED_WARP: one ray per warp for frames of any size, each warp taking
  *     32 rays of its tile one after another, records in shared memory (measured
  *     slower on large aerial views: rays of one tile are marched one after
@@ -667,9 +668,10 @@ cow_status cow_set_schedule(cow_ctx *ctx, int32_t schedule);
  * over 2x2 blocks of 128^3 / 512^2 FP32 features: forward 39.9 -> 28.3 ms).
  * COW_RAY_ORDER_GIVEN: warp t marches ray t.  Rays that are mostly alike their
  * neighbours (a camera's) are marched one ray per thread in the given order,
- * from 8000 + 280 P rays up (at most 2^17); a key pass counts the alike ones.
- * Random rays are marched one ray per thread in calls so large that many meet in
- * a texel.  Both but for the backwards and most opacity gradients, which are
+ * from 8000 + 280 P rays up (at most 2^17; with unbounded blocks 11000 + 45 P, at
+ * most 20000); a key pass counts the alike ones.  Random rays are marched one ray
+ * per thread in calls so large that many meet in a texel, and through unbounded
+ * blocks from 24000 + 170 P rays up (at most 45000).  Both but for the backwards and most opacity gradients, which are
  * faster one ray per warp.
  * Outputs are written at each ray's own index either way and each ray's values
  * are the same; gradient sums change only by the order of their FP32

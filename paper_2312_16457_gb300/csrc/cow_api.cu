@@ -617,11 +617,16 @@ int32_t forced_form(const cow_ctx *c) {
 struct CallShape {
     int32_t n_ids;
     int64_t P;  // the smallest plane resolution of the call's blocks: lattice points across a block
+    bool unbounded;  // any contracted block
 };
 
 CallShape call_shape(const cow_ctx *c, const int32_t *ids, int32_t n_ids) {
-    CallShape s = {n_ids, n_ids > 0 ? INT32_MAX : 0};
-    for (int32_t k = 0; k < n_ids; k++) s.P = std::min<int64_t>(s.P, c->blocks[(size_t)ids[k]].P);
+    CallShape s = {n_ids, n_ids > 0 ? INT32_MAX : 0, false};
+    for (int32_t k = 0; k < n_ids; k++) {
+        const BlockHost &b = c->blocks[(size_t)ids[k]];
+        s.P = std::min<int64_t>(s.P, b.P);
+        s.unbounded |= b.unb != 0;
+    }
     return s;
 }
 
@@ -631,7 +636,12 @@ CallShape call_shape(const cow_ctx *c, const int32_t *ids, int32_t n_ids) {
 // Pixels at which both took the same (FP32 / BF16, one, four and sixteen
 // blocks): P = 32 19 k; P = 64 33, 32, 35 k; P = 96 44, 42, 50 k; P = 128 58, 43
 // (FP16 62), 60 k; P = 192 -, 62 (FP16 70), 75 k; P = 256 85 k; P = 512 -, -, 140 k.
-int64_t warp_pixels(const CallShape &s) { return 8000 + 280 * s.P; }
+// Contracted blocks: t advances by each point's own step, so every lane of a
+// warp walks all points of its scan, and empty space has no jump; four of them,
+// FP32 / BF16: P = 32 12 / 11 k, P = 96 18 / 15 k, P = 256 24 / 18 k, P = 512 26 / 20 k.
+int64_t warp_pixels(const CallShape &s) {
+    return s.unbounded ? std::min<int64_t>(20000, 11000 + 45 * s.P) : 8000 + 280 * s.P;
+}
 
 // At most kChipRays pixels, which one ray per thread has on the chip at once.
 // Measured (us, thread / warp form): M = 1 block of 64^3 and 256^2 FP32, 128x128
@@ -672,10 +682,14 @@ enum RayCall { kCallMarch, kCallPartials, kCallOpacity, kCallOpacityGrad, kCallO
 //   16     32    320 / 330    150 / 78     180 / 85
 //   16     64    2600 / 2600  530 / 150    - / 340
 // and 2.56 M rays, the most measured, left the warp form ahead at "-".
+// Four contracted blocks (warp_pixels), march 35 / 30, 48 / 40, 56 / 43, 65 / 44 at
+// P = 32, 96, 256, 512, partials and opacity up to a quarter less.
 int64_t thread_rays(const cow_ctx *c, const CallShape &s, RayCall call) {
     const bool f32 = c->dtype == cow::kF32;
     const double P = (double)s.P, n = s.n_ids;
     double rays = 1e18;
+    if (s.unbounded && (call == kCallOpacityGrad || call == kCallOpacityGradT)) return INT64_MAX;
+    if (s.unbounded) return std::min<int64_t>(45000, 24000 + 170 * s.P);
     switch (call) {
         case kCallMarch:
             rays = n == 1 ? (f32 ? std::max(600 * P, 13 * P * P) : 450 * P)

@@ -294,3 +294,31 @@ def test_small_planes_take_the_thread_form_earlier():
         ctx.sync_check()
         ctx.close()
     assert form == {(k, P): "thread" if P == 33 else "warp" for P in (33, 260) for k in ("view", "camera", "random")}
+
+
+def test_unbounded_blocks_take_the_thread_form_earlier():
+    """Contracted blocks: frames and batches from some 20000 rays on."""
+    mlp = torch.from_numpy(synth.mlp_weights(9)).cuda()
+    sc, cams, _ = synth.workload_unbounded(R=9, P=260)
+    form = {}
+    for flags in (True, False):
+        ctx = cow.Context(sc, "bf16")
+        if not flags:
+            for i in IDS:
+                ctx.set_unbounded(i, 0)
+        for w, h in ((120, 100), (250, 200)):
+            cam = synth.Camera(cams[0].c2w, w, h, 70.0)
+            ctx.render([cam], [ctx.sort_blocks(cam, IDS)], mlp)
+            form["view", flags, w] = ctx.last_form()
+            o, d = (torch.from_numpy(x).cuda() for x in oracle.pixel_rays(cam))
+            perm = torch.randperm(w * h, generator=torch.Generator().manual_seed(1)).cuda()
+            o, d = o[perm], d[perm]
+            for name, call in (("march", lambda: ctx.render_rays(o, d, IDS, mlp)),
+                               ("partials", lambda: ctx.render_partials(o, d, IDS)),
+                               ("opacity", lambda: ctx.opacity_loss(o, d, IDS))):
+                call()
+                form[name, flags, w] = ctx.last_form()
+        ctx.sync_check()
+        ctx.close()
+    assert form == {(k, u, w): "thread" if u and w == 250 else "warp" for k in ("view", "march", "partials", "opacity")
+                    for u in (True, False) for w in (120, 250)}
