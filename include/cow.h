@@ -671,8 +671,8 @@ cow_status cow_set_schedule(cow_ctx *ctx, int32_t schedule);
  * from 8000 + 280 P rays up (at most 2^17; with unbounded blocks 11000 + 45 P, at
  * most 20000); a key pass counts the alike ones.  Random rays are marched one ray
  * per thread in calls so large that many meet in a texel, and through unbounded
- * blocks from 24000 + 170 P rays up (at most 45000).  Both but for the backwards and most opacity gradients, which are
- * faster one ray per warp.
+ * blocks from 24000 + 170 P rays up (at most 45000).  Both but for the backwards and the opacity
+ * gradient's scatter, which are faster one ray per warp.
  * Outputs are written at each ray's own index either way and each ray's values
  * are the same; gradient sums change only by the order of their FP32
  * reductions.  The coherent order costs a key pass, a scan and a scatter, about

@@ -576,6 +576,13 @@ __global__ void __launch_bounds__(kBwdThreads) k_sparsity(RegArgs a, const __gri
     if (threadIdx.x == 0 && a.loss) atomicAdd(a.loss, term);
 }
 
+// One (ray, block)'s share of the loss, from alpha^k.
+constexpr float kAlphaEps = 1e-6f;
+__device__ __forceinline__ float opacity_term(const RegArgs &a, float a_raw) {
+    const float al = fminf(fmaxf(a_raw, kAlphaEps), 1.f - kAlphaEps);
+    return -(a.weight / (float)a.n_rays) * (al * logf(al) + (1.f - al) * log1pf(-al));
+}
+
 // Opacity, one ray per warp.  Bound by the L2's scattered reductions (65537 BF16
 // rays: a step of 8.4 ms, 12.1 ms with one ray per thread and 20 reductions a
 // sample).
@@ -587,8 +594,11 @@ __global__ void __launch_bounds__(kBwdThreads, COW_REG_MIN_BLOCKS) k_opacity(con
     WarpScratch &ws = bs.w;
     const int lane = threadIdx.x & 31;
     float term = 0.f;
-    const float scale = a.weight / (float)a.n_rays, eps = 1e-6f;
-    const int64_t n_rays = rays_alike(a) ? 0 : a.n_rays;  // alike: k_opacity_t has them
+    const float scale = a.weight / (float)a.n_rays, eps = kAlphaEps;
+    bool given;
+    const bool marched = thread_form(a, given);  // by k_opacity_t: into out_T, or to the term itself
+    const int64_t n_rays = marched && !a.out_T ? 0 : a.n_rays;
+    const float *block_T = marched ? a.out_T : a.block_T;
     for (int64_t ray = first_ray(); ray < n_rays; ray += (int64_t)gridDim.x * kBwdWarps) {
         float o[3], d[3], inv_d[3], omax;
         const int64_t r = load_ray_warp(a, ray, o, d);
@@ -599,8 +609,8 @@ __global__ void __launch_bounds__(kBwdThreads, COW_REG_MIN_BLOCKS) k_opacity(con
             const int pos = ws.ord[k], id = rr.id[pos];
             const BlockRec &b = rr.r[pos];
             float T = 1.f;
-            if (a.block_T) {  // the forward's in-block transmittance
-                T = __ldg(a.block_T + r * rr.n + pos);
+            if (block_T) {  // the forward's in-block transmittance, or k_opacity_t's
+                T = __ldg(block_T + r * rr.n + pos);
                 if (T < 0.f) return true;  // no occupied sample
             } else {
                 int nk = 0;
@@ -621,7 +631,7 @@ __global__ void __launch_bounds__(kBwdThreads, COW_REG_MIN_BLOCKS) k_opacity(con
             }
             const float a_raw = 1.f - T;
             const float al = fminf(fmaxf(a_raw, eps), 1.f - eps);
-            term -= scale * (al * logf(al) + (1.f - al) * log1pf(-al));
+            term += opacity_term(a, a_raw);
             if (!a.grad_grid || !(a_raw > eps && a_raw < 1.f - eps)) return true;
             const float ga = -scale * (logf(al) - log1pf(-al));  // d loss / d alpha^k
             float *const gp[3] = {a.grad_planes[3 * id], a.grad_planes[3 * id + 1], a.grad_planes[3 * id + 2]};
@@ -644,13 +654,13 @@ __global__ void __launch_bounds__(kBwdThreads, COW_REG_MIN_BLOCKS) k_opacity(con
     if (threadIdx.x == 0) a.loss_parts[blockIdx.x] = term;
 }
 
-// The same, one ray per thread (ray_form in cow_api.cu), every sample
-// scattered by its own thread; the loss's parts behind k_opacity's.
+// Its first march, one ray per thread (ray_form in cow_api.cu): the blocks' own
+// transmittances go to out_T, for k_opacity to scatter from, or, without a
+// gradient, the term is taken at once, its parts behind k_opacity's.
 template <int DT>
 __global__ void __launch_bounds__(kBwdThreads, COW_REG_MIN_BLOCKS) k_opacity_t(const __grid_constant__ RegArgs a,
                                                                             const __grid_constant__ RayRecs rr) {
     float term = 0.f;
-    const float scale = a.weight / (float)a.n_rays, eps = 1e-6f;
     bool given;
     const int64_t n_rays = thread_form(a, given) ? a.n_rays : 0;
     for (int64_t ray = (int64_t)blockIdx.x * kBwdThreads + threadIdx.x; ray < n_rays;
@@ -658,46 +668,25 @@ __global__ void __launch_bounds__(kBwdThreads, COW_REG_MIN_BLOCKS) k_opacity_t(c
         float o[3], d[3], inv_d[3], omax;
         const int64_t r = load_ray(a, ray, given, o, d);
         ray_setup(d, o, inv_d, omax);
-        int order[kMaxRayIds];
-        const int n = sort_blocks_for_ray(rr, o, order);
-        for (int k = 0; k < n; k++) {
-            const int pos = order[k], id = rr.id[pos];
-            const BlockRec &b = rr.r[pos];
-            float T = 1.f;
-            if (a.block_T) {
-                T = __ldg(a.block_T + r * rr.n + pos);
-                if (T < 0.f) continue;
-            } else {
-                int nk = 0;
-                DepthSum tau;
-                BrickCache bc;
-                for_each_sample(b, o, d, inv_d, omax, a.err,
-                                [&](const float *, const float rel[3], const float g[3], float delta) {
-                    float2 f2[4];
-                    accumulate_sample<DT>(b, rel, g, f2, &bc);
-                    tau.add(expf(f2[0].x) * delta);
-                    nk++;
-                    return true;
-                });
-                if (nk == 0) continue;
-                T = tau.transmittance();
-            }
-            const float a_raw = 1.f - T;
-            const float al = fminf(fmaxf(a_raw, eps), 1.f - eps);
-            term -= scale * (al * logf(al) + (1.f - al) * log1pf(-al));
-            if (!a.grad_grid || !(a_raw > eps && a_raw < 1.f - eps)) continue;
-            const float ga = -scale * (logf(al) - log1pf(-al));
-            float *const gp[3] = {a.grad_planes[3 * id], a.grad_planes[3 * id + 1], a.grad_planes[3 * id + 2]};
+        for (int k = 0; k < rr.n; k++) {
+            const BlockRec &b = rr.r[k];
+            int nk = 0;
+            DepthSum tau;
             BrickCache bc;
             for_each_sample(b, o, d, inv_d, omax, a.err,
                             [&](const float *, const float rel[3], const float g[3], float delta) {
                 float2 f2[4];
                 accumulate_sample<DT>(b, rel, g, f2, &bc);
-                scatter_ch0(b, a.grad_grid[id], gp, rel, g, ga * expf(f2[0].x) * delta * T);
+                tau.add(expf(f2[0].x) * delta);
+                nk++;
                 return true;
             });
+            const float T = nk ? tau.transmittance() : -1.f;
+            if (a.out_T) a.out_T[r * rr.n + k] = T;
+            else if (nk) term += opacity_term(a, 1.f - T);
         }
     }
+    if (a.out_T) return;
     term = cta_sum(term);
     if (threadIdx.x == 0) a.loss_parts[kOpacityMaxCtas + blockIdx.x] = term;
 }
@@ -1086,16 +1075,16 @@ cudaError_t launch_opacity(const RegArgs &a, const RayRecs &rr, cudaStream_t st)
     const auto ctas = [&](int rays) {
         return (unsigned)std::min<int64_t>((a.n_rays + rays - 1) / rays, kOpacityMaxCtas);
     };
-    // as launch_rays_dt: with a count of alike rays both are launched
-    const unsigned nw = a.form == kFormWarp ? ctas(kBwdWarps) : 0;
+    // as launch_rays_dt: with a count of alike rays the device decides
     const unsigned nt = a.form == kFormThread || a.ray_alike ? ctas(kBwdThreads) : 0;
+    const unsigned nw = a.form == kFormWarp || a.out_T ? ctas(kBwdWarps) : 0;
     const cudaError_t e_ = dispatch_dt(a.dtype, [&](auto D) {
         if (nt) k_opacity_t<decltype(D)::value><<<nt, kBwdThreads, 0, st>>>(a, rr);
         if (nw) k_opacity<decltype(D)::value><<<nw, kBwdThreads, 0, st>>>(a, rr);
         return cudaSuccess;
     });
     if (e_ != cudaSuccess) return e_;
-    if (a.loss) k_add_parts<<<1, 1024, 0, st>>>(a.loss_parts, (int)nw, (int)nt, a.loss);
+    if (a.loss) k_add_parts<<<1, 1024, 0, st>>>(a.loss_parts, (int)nw, a.out_T ? 0 : (int)nt, a.loss);
     return cudaGetLastError();
 }
 

@@ -656,9 +656,12 @@ int32_t view_form(const cow_ctx *c, const int32_t *ids, int32_t n_ids, int64_t n
 }
 
 // What a ray batch is marched for: the outputs of the march, the block-parallel
-// form's partials, the opacity term, the term and its gradient (which marches
-// every block twice), the gradient from the forward's in-block transmittances.
-enum RayCall { kCallMarch, kCallPartials, kCallOpacity, kCallOpacityGrad, kCallOpacityGradT };
+// form's partials, the in-block opacity (the regulariser's term, or the first of
+// its gradient's two marches).  What scatters gradients runs one ray per warp:
+// its sums over the samples of a voxel are faster to reduce and lose less than
+// single samples added to a large sum (90 k camera rays over contracted blocks,
+// density gradient of the nearest: 1.4e-3 of its largest entry lost).
+enum RayCall { kCallMarch, kCallPartials, kCallOpacity };
 
 // Random rays from which one ray per thread is the faster form.  It pays where
 // many rays meet in few texels, so that the rays of a warp (sorted, ray_order.cu)
@@ -666,8 +669,7 @@ enum RayCall { kCallMarch, kCallPartials, kCallOpacity, kCallOpacityGrad, kCallO
 // the blocks, between which rays diverge, and with the bytes of an FP32 texel.
 // Small storage stays in L1 and L2 when one block or the partials of one block at
 // a time are marched; there the longest ray, some P samples, decides.  The
-// opacity term reads and composites less a sample, which suits the warp form, as
-// does the gradient's scatter, but for many blocks of few samples each.
+// opacity reads and composites less a sample, which suits the warp form.
 // Thousands of rays at which both took the same, FP32 / BF16:
 //   blocks P     march        partials     opacity
 //    1     32    20 / 14      28 / 18      18 / 15
@@ -688,7 +690,6 @@ int64_t thread_rays(const cow_ctx *c, const CallShape &s, RayCall call) {
     const bool f32 = c->dtype == cow::kF32;
     const double P = (double)s.P, n = s.n_ids;
     double rays = 1e18;
-    if (s.unbounded && (call == kCallOpacityGrad || call == kCallOpacityGradT)) return INT64_MAX;
     if (s.unbounded) return std::min<int64_t>(45000, 24000 + 170 * s.P);
     switch (call) {
         case kCallMarch:
@@ -700,10 +701,6 @@ int64_t thread_rays(const cow_ctx *c, const CallShape &s, RayCall call) {
             if (f32 ? P <= 48 || (n == 1 && P <= 64) : P <= 128 || (n == 1 && P <= 192))
                 rays = f32 ? P * P * P * (0.3 + 0.35 * n) : P * P * 5 * (1 + n);
             break;
-        case kCallOpacityGrad:
-            if (n > 8 && P <= 64) rays = 5000 * P;  // 16 blocks, P = 32, 1.28 M rays: 0.57 to 0.70 of the warp form's time
-            break;
-        case kCallOpacityGradT: break;
     }
     return (int64_t)std::min(rays, 1e18);
 }
@@ -711,14 +708,8 @@ int64_t thread_rays(const cow_ctx *c, const CallShape &s, RayCall call) {
 // A camera's rays from which one ray per thread, in the given order, is the
 // faster form.  921600 of them (ms, thread / warp): 16 blocks of 128^3 and 512^2
 // FP16, march 8.7 / 13.4, with in-block transmittances 9.9 / 13.7, partials 9.5 /
-// 12.0, opacity 7.3 / 10.6, with its gradient 29.6 / 29.5 and, from the
-// transmittances, 24.2 / 21.1; 10^6 through 16 blocks of 96^2 FP32, opacity and
-// gradient 13.4 / 16.4.
-int64_t thread_alike(const CallShape &s, RayCall call) {
-    if (call == kCallOpacityGradT || (call == kCallOpacityGrad && s.n_ids <= 8)) return INT64_MAX;
-    if (call == kCallOpacityGrad) return 2000 * s.P;
-    return std::min(warp_pixels(s), cow::kRaysAlikeMin);
-}
+// 12.0, opacity 7.3 / 10.6.
+int64_t thread_alike(const CallShape &s) { return std::min(warp_pixels(s), cow::kRaysAlikeMin); }
 
 // The form of a ray batch.  *count: the device counts the alike rays, and takes
 // the thread form in the given order when it is a camera's.
@@ -728,7 +719,7 @@ int32_t ray_form(const cow_ctx *c, const int32_t *ids, int32_t n_ids, int64_t n,
     const CallShape s = call_shape(c, ids, n_ids);
     const int32_t form = n >= thread_rays(c, s, call) ? cow::kFormThread : cow::kFormWarp;
     // a call in the thread form asks only whether to keep to the given order
-    *count = n >= thread_alike(s, call) && (form == cow::kFormWarp || c->ray_order == COW_RAY_ORDER_COHERENT);
+    *count = n >= thread_alike(s) && (form == cow::kFormWarp || c->ray_order == COW_RAY_ORDER_COHERENT);
     return form;
 }
 
@@ -1629,9 +1620,21 @@ cow_status cow_opacity_loss(cow_ctx *ctx, const float *o, const float *d, int64_
     a.weight = weight;
     a.block_T = block_T;
     a.loss_parts = (float *)(ctx->d_err + kCtxLossParts);
-    bool count;
-    const RayCall call = !grad_grid ? kCallOpacity : block_T ? kCallOpacityGradT : kCallOpacityGrad;
-    a.form = ray_form(ctx, ids, n_ids, n_rays, call, &count);
+    bool count = false;
+    a.form = block_T ? cow::kFormWarp : ray_form(ctx, ids, n_ids, n_rays, kCallOpacity, &count);
+    if (!block_T && grad_grid && (count || a.form == cow::kFormThread)) {
+        // the first march's transmittances; without room for them, and in a capture (a
+        // later call may free them), both marches run one ray per warp
+        cudaStreamCaptureStatus cs = cudaStreamCaptureStatusNone;
+        if (cudaStreamIsCapturing(st, &cs) == cudaSuccess && cs == cudaStreamCaptureStatusNone &&
+            ctx->bm_scratch.reserve((size_t)n_rays * (size_t)n_ids * sizeof(float)) == cudaSuccess) {
+            a.out_T = (float *)ctx->bm_scratch.p;
+        } else {
+            cudaGetLastError();
+            a.form = cow::kFormWarp;
+            count = false;
+        }
+    }
     if ((rc = ray_order(ctx, o, d, n_rays, ids, n_ids, st, &a.ray_perm, count, &a.ray_alike)) != COW_OK) return rc;
     cow::RayRecs rr;
     make_ray_recs(ctx, ids, n_ids, rr);

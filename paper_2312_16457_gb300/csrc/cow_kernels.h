@@ -140,6 +140,8 @@ struct RegArgs {                  // the blocks that take part come by value (Ra
     float weight;                 // the loss and its gradient are scaled by weight / n_rays
     const float *block_T;         // opacity: the forward's n_rays x n_ids in-block transmittances (-1: no
                                   // sample), or null to march every block twice
+    float *out_T;                 // opacity with a gradient, without block_T: scratch for the same, when the first
+                                  // march may run one ray per thread
     float *loss;                  // device float, accumulated (may be null)
     float *loss_parts;            // opacity: scratch, 2 kOpacityMaxCtas floats
     float *const *grad_grid;      // device pointer table as in BwdArgs (null: no gradient)

@@ -124,18 +124,20 @@ def _rays(opt, sc, n):
 
 
 def _marches(ctx, sc, o, d, mlp, ids):
-    """Every ray call that chooses a form: (calls, opacity gradients)."""
+    """Every ray call that chooses a form: (the form, outputs, in-block
+    transmittances, opacity gradients)."""
     out = list(ctx.render_rays(o, d, ids, mlp, ert_eps=1e-2, nsamp=True))
     out += list(ctx.render_rays(o, d, ids, None, ert_eps=1e-2, nsamp=True, block_mlps=True))
     out += [*ctx.render_rays_block_t(o, d, ids, mlp)[:2], *ctx.render_rays_block_state(o, d, ids)]
     out.append(ctx.render_partials(o, d, ids))
+    form = ctx.last_form()
     bt = ctx.render_rays_block_t(o, d, ids, mlp)[2]
     grads = []
     for T in (None, bt):
         gg = [torch.zeros(b.grid.shape, device="cuda") for b in sc.blocks]
         gp = [[torch.zeros(p.shape, device="cuda") for p in b.planes] for b in sc.blocks]
         grads.append([ctx.opacity_loss(o, d, ids, 0.5, grads=(gg, gp), block_T=T), *gg, *sum(gp, [])])
-    return out, bt, grads
+    return form, out, bt, grads
 
 
 @pytest.mark.parametrize("form", FORMS)
@@ -153,10 +155,10 @@ def test_ray_calls_do_not_depend_on_the_form(form):
     for f in ("thread", "warp"):
         ctx.set_test_hooks(form=f)
         res.append(_marches(ctx, sc, o, d, mlp, IDS))
-        assert ctx.last_form() == f
+        assert res[-1][0] == f
     ctx.set_test_hooks()
     ctx.sync_check()
-    (a, bt_a, ga), (b, bt_b, gb) = res
+    (_, a, bt_a, ga), (_, b, bt_b, gb) = res
     for x, y in zip(a, b):
         assert torch.equal(x, y)
     assert torch.equal(bt_a < 0, bt_b < 0) and int((bt_a >= 0).sum()) > 500
@@ -322,3 +324,41 @@ def test_unbounded_blocks_take_the_thread_form_earlier():
         ctx.close()
     assert form == {(k, u, w): "thread" if u and w == 250 else "warp" for k in ("view", "march", "partials", "opacity")
                     for u in (True, False) for w in (120, 250)}
+
+
+@pytest.mark.parametrize("order", ["coherent", "given"])
+def test_opacity_gradient_with_a_thread_form_first_march(order):
+    """A camera's rays: the transmittances of the first march come from the thread
+    form, the scatter runs one ray per warp.  The same loss and gradient as from
+    the forward's transmittances, summed in 64 bits over 64 calls."""
+    sc = synth.city_scene(23, 2, 2.0, [(66, 260)], **synth.SPARSE_CITY)
+    mlp = torch.from_numpy(synth.mlp_weights(9)).cuda()
+    ctx = cow.Context(sc, "bf16")
+    ctx.set_ray_order(order)
+    o, d = _camera_rays(500, 301)
+    n = o.shape[0]
+
+    def term(part, T):
+        gg = [torch.zeros(b.grid.shape, device="cuda") for b in sc.blocks]
+        gp = [[torch.zeros(p.shape, device="cuda") for p in b.planes] for b in sc.blocks]
+        k = o[part].shape[0]
+        loss = ctx.opacity_loss(o[part], d[part], IDS, weight=k / n, grads=(gg, gp), block_T=T)
+        return [loss, *gg, *sum(gp, [])]
+
+    got = term(slice(None), None)
+    assert ctx.last_form() == "thread"
+    ctx.set_test_hooks(form="thread")
+    T, want = ctx.render_rays_block_t(o, d, IDS, mlp)[2], None
+    for k in range(64):
+        part = slice(k * n // 64, (k + 1) * n // 64)
+        x = [y.double() for y in term(part, T[part].contiguous())]
+        assert ctx.last_form() == "warp"
+        want = x if want is None else [a + b for a, b in zip(want, x)]
+    ctx.sync_check()
+    # T of both marches: expf against __expf of the log-density and its product, some
+    # 1e-6 tau relative; where T nears the clamp at 1e-6 (tau = 14) the gradient's
+    # log(1 - alpha) and its rounding take up to 1e-2 of a single ray's share, the
+    # largest entry sums hundreds of rays
+    for a, b in zip(got, want):
+        assert float((a.double() - b).abs().max()) <= 1e-3 * float(b.abs().max())
+    ctx.close()
