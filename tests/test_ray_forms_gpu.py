@@ -362,3 +362,21 @@ def test_opacity_gradient_with_a_thread_form_first_march(order):
     for a, b in zip(got, want):
         assert float((a.double() - b).abs().max()) <= 1e-3 * float(b.abs().max())
     ctx.close()
+
+
+@pytest.mark.parametrize("ert", [0.0, 1e-2])
+@pytest.mark.parametrize("storage", ["fp32", "fp8_bf16d"])
+def test_warp_schedule_of_odd_frames(storage, ert):
+    """COW_SCHED_WARP: warps whose 32 pixels lie partly outside the frame."""
+    ctx = cow.Context(_city(), storage)
+    res = []
+    cams = [synth.camera((-2.6, -3.1, 2.0), (0.3, 0.2, -0.8), w, h, 60.0) for w, h in ((37, 29), (1, 1), (16, 9))]
+    ids = [ctx.sort_blocks(c, IDS) for c in cams]
+    for sched, form in (("thread", "thread"), ("warp", "warp")):
+        ctx.set_schedule(sched)
+        res.append(ctx.render(cams, ids, synth.mlp_weights(9), ert_eps=ert, nsamp=True))
+        assert ctx.last_form() == form
+    ctx.sync_check()
+    for x, y in zip(*res):
+        assert torch.equal(x, y)
+    ctx.close()
