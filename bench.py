@@ -656,10 +656,10 @@ def run_fit(args, ws, rank, local):
     ms = float(np.mean([a.elapsed_time(b) for a, b in evs]))
     p1 = psnr_now()
     n = o.shape[0]
-    # the backward alone (K7 + the K6 re-march), against the measured rate of
-    # random non-returning float4 reductions into an L2-resident buffer: K6
-    # scatters 2 float4 reductions to each of the 20 taps of every occupied
-    # sample
+    # the backward alone (K7 + the K6 re-march): 40 float4 contributions to its 20
+    # taps for every occupied sample, which K6 adds up per voxel and texel cell
+    # before it reduces them; beside it the measured rates of random
+    # non-returning float4 reductions
     bwd = None
     if not per_block and not args.reg:
         rgb, aux, ns = fit.ctx.render_rays(o, d, fit.ids, fit.mlp, nsamp=True)
@@ -673,20 +673,19 @@ def run_fit(args, ws, rank, local):
                         stream)
         fit.ctx.sync_check()
         samples = int(ns.to(torch.int64).sum().item())
-        reds = 40 * samples
+        contributions = 40 * samples
         ms_b = float(np.mean(tb))
         peak_red = cow.reduce_peak(32 << 20)
         peak_red_hbm = cow.reduce_peak(8 << 30, iters=64)
-        rate = reds / (ms_b / 1000.0) / 1e9
-        bwd = {"ms": round(ms_b, 3), "occupied_samples": samples, "float4_reductions": reds,
-               "achieved_gred_per_s": round(rate, 2),
-               "peak_gred_per_s_l2": round(peak_red, 2), "frac_of_l2_reduce_peak": round(rate / peak_red, 3),
-               "peak_gred_per_s_hbm": round(peak_red_hbm, 2),
+        rate = contributions / (ms_b / 1000.0) / 1e9
+        bwd = {"ms": round(ms_b, 3), "occupied_samples": samples, "float4_contributions": contributions,
+               "gcontributions_per_s": round(rate, 2),
+               "peak_gred_per_s_l2": round(peak_red, 2), "peak_gred_per_s_hbm": round(peak_red_hbm, 2),
                "peak_source": "measured live: random red.global.add.v4.f32 into a 32 MiB (L2-resident) buffer, "
                               "cow_reduce_peak",
-               "note": "time of the whole backward call (MLP backward + re-march); reductions counted as the 40 "
-                       "float4 contributions of an occupied sample: the kernel adds up those of one voxel or "
-                       "texel cell and reduces in 64-byte groups, so the rate can exceed the probe's"}
+               "note": "time of the whole backward call (MLP backward + re-march); the kernel adds up the "
+                       "contributions to one voxel or texel cell and reduces in 64-byte groups, so their rate is "
+                       "not the reductions' and can exceed the probe's"}
     line = {"metric": "differentiation form: training rays/s (forward + backward + Adam)", "value": round(n / ms / 1e3, 3),
             "unit": "Mrays/s", "n_gpus": ws, "steps": args.steps, "warmup": args.warmup, "ms_per_step": round(ms, 3),
             "higher_is_better": True, "dtype": "f32", "data": "synthetic",
