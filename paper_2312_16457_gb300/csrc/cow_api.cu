@@ -568,7 +568,7 @@ void make_ray_recs(const cow_ctx *c, const int32_t *ids, int32_t n, cow::RayRecs
 // box.  The permutation lives in the context until the next call.  With
 // `count`, *alike receives where the count of alike neighbours will be.  The
 // given order uses no buffer that grows (a graph captured from such a call
-// must outlive every later call's sizes): its count is one of the words
+// must outlive every later call's sizes): the count is one of the words
 // allocated with the context, each call's the next one, so that calls on
 // several streams do not share it.
 constexpr int64_t kRayOrderMin = 8192;
@@ -587,19 +587,18 @@ cow_status ray_order(cow_ctx *c, const float *o, const float *d, int64_t n, cons
             hi[a] = std::max(hi[a], b.hi[a]);
         }
     }
+    uint32_t *n_alike = count ? c->d_err + cowi::kCtxAlike + c->alike_word++ % cowi::kCtxAlikeWords : nullptr;
+    if (alike) *alike = n_alike;
     if (!sort) {
-        uint32_t *n_alike = c->d_err + cowi::kCtxAlike + c->alike_word++ % cowi::kCtxAlikeWords;
         COW_CUDA(cow::launch_count_alike(o, d, n, lo, hi, n_alike, st));
-        *alike = n_alike;
         return COW_OK;
     }
     COW_CUDA(c->ray_keys.reserve((size_t)n * sizeof(uint32_t)));
     COW_CUDA(c->ray_hist.reserve((size_t)cow::kRayOrderHistWords * sizeof(uint32_t)));
     COW_CUDA(c->ray_perm.reserve((size_t)n * sizeof(int32_t)));
     COW_CUDA(cow::launch_ray_order(o, d, n, lo, hi, (uint32_t *)c->ray_keys.p, (uint32_t *)c->ray_hist.p,
-                                   (int32_t *)c->ray_perm.p, st));
+                                   (int32_t *)c->ray_perm.p, n_alike, st));
     *perm = (const int32_t *)c->ray_perm.p;
-    if (count) *alike = (const uint32_t *)c->ray_hist.p + cow::kRayOrderAlike;
     return COW_OK;
 }
 
@@ -707,8 +706,8 @@ int64_t thread_rays(const cow_ctx *c, const CallShape &s, RayCall call) {
 
 // A camera's rays from which one ray per thread, in the given order, is the
 // faster form.  921600 of them (ms, thread / warp): 16 blocks of 128^3 and 512^2
-// FP16, march 8.7 / 13.4, with in-block transmittances 9.9 / 13.7, partials 9.5 /
-// 12.0, opacity 7.3 / 10.6.
+// FP16, march 8.7 / 13.4, with in-block transmittances 9.5 / 13.7, partials 9.2 /
+// 12.0, opacity 6.4 / 10.6.
 int64_t thread_alike(const CallShape &s) { return std::min(warp_pixels(s), cow::kRaysAlikeMin); }
 
 // The form of a ray batch.  *count: the device counts the alike rays, and takes

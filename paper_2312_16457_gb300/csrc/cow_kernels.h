@@ -38,8 +38,8 @@ struct MarchArgs {
     float *out_partials;             // block-parallel form: n_rays x n_ids x 8 per-block partials (written)
     const float *in_partials;        // block-parallel form: the same, read by the compositor
     const int32_t *ray_perm;         // ray mode, may be null: ray t of the order is ray ray_perm[t] (outputs at the ray's index)
-    const uint32_t *ray_alike;       // ray mode, kFormWarp, may be null: rays whose order key is the next ray's; the
-                                     // device takes kFormThread in the given order when most are (rays_alike)
+    const uint32_t *ray_alike;       // ray mode, may be null: rays whose order key is the next ray's; when most are
+                                     // (rays_alike) the device takes kFormThread, in the given order
     float *out_block_state;          // ray mode, per-block MLPs, may be null: n_rays x n_ids x 8, per (ray, block
                                      // at its position in ids) C^k (3), F^k (4), the transmittance in front (-1: no sample)
 };
@@ -56,7 +56,7 @@ constexpr int64_t kChipRays = kSms * 512;
 constexpr uint32_t kTestSkipRecordCopy = 1u;
 
 // marching schedules of the view kernel
-constexpr int kSchedWarp = 0;         // one ray per warp, lanes on consecutive lattice samples
+constexpr int kSchedWarp = 0;         // one ray per warp, a tile's rays one after another
 constexpr int kSchedThread = 1;       // one ray per thread, records in shared memory
 constexpr int kSchedThreadConst = 2;  // one ray per thread, records in the parameter buffer
 struct ParamRecs;
@@ -67,8 +67,8 @@ cudaError_t launch_march_rays(const MarchArgs &a, const RayRecs &rr, cudaStream_
 // marches, grouping rays by the cells of their entry into the box [lo, hi]
 // and their exit from it.  keys: n scratch words; hist: kRayOrderHistWords
 // words (the bins; at kRayOrderAlike the count of rays whose key is the next
-// ray's; the totals of the scan's blocks of 1024 bins).  launch_count_alike:
-// the count alone, in its own word.
+// ray's; the totals of the scan's blocks of 1024 bins).  n_alike: the count's own
+// word, may be null.  launch_count_alike: the count alone.
 constexpr int kRayOrderKeyBits = 20;
 constexpr int kRayOrderBins = 1 << kRayOrderKeyBits;
 constexpr int kRayOrderAlike = kRayOrderBins;
@@ -79,7 +79,7 @@ constexpr int64_t kRaysAlikeMin = 1 << 17;
 // Whether n of a call's n_rays rays, alike the next one, make it a camera's.
 __host__ __device__ __forceinline__ bool mostly_alike(uint32_t n, int64_t n_rays) { return 4 * (int64_t)n >= 3 * n_rays; }
 cudaError_t launch_ray_order(const float *o, const float *d, int64_t n, const float lo[3], const float hi[3],
-                             uint32_t *keys, uint32_t *hist, int32_t *perm, cudaStream_t st);
+                             uint32_t *keys, uint32_t *hist, int32_t *perm, uint32_t *n_alike, cudaStream_t st);
 cudaError_t launch_count_alike(const float *o, const float *d, int64_t n, const float lo[3], const float hi[3],
                                uint32_t *n_alike, cudaStream_t st);
 // Block-parallel form: per-block partials of a ray batch (8 floats per ray

@@ -148,7 +148,9 @@ __global__ void __launch_bounds__(kScanBlocks) k_scan_sums(uint32_t *sums) {
 }
 
 __global__ void k_ray_scatter(const uint32_t *__restrict__ keys, int64_t n, uint32_t *__restrict__ offs,
-                              const uint32_t *__restrict__ sums, int32_t *__restrict__ perm) {
+                              const uint32_t *__restrict__ sums, int32_t *__restrict__ perm,
+                              uint32_t *n_alike) {
+    if (n_alike && blockIdx.x == 0 && threadIdx.x == 0) *n_alike = offs[kRayOrderAlike];  // behind the bins
     for (int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; i < n; i += (int64_t)gridDim.x * blockDim.x) {
         const uint32_t k = keys[i];
         perm[sums[k / kScanThreads] + atomicAdd(offs + k, 1u)] = (int32_t)i;
@@ -182,7 +184,7 @@ int key_blocks(int64_t n) { return (int)std::min<int64_t>((n + 255) / 256, kSms 
 }  // namespace
 
 cudaError_t launch_ray_order(const float *o, const float *d, int64_t n, const float lo[3], const float hi[3],
-                             uint32_t *keys, uint32_t *hist, int32_t *perm, cudaStream_t st) {
+                             uint32_t *keys, uint32_t *hist, int32_t *perm, uint32_t *n_alike, cudaStream_t st) {
     static_assert(kRayOrderBins == kScanBlocks * kScanThreads && kScanBlocks <= 1024 && kScanBlocks % 32 == 0,
                   "two-level scan shape");
     static_assert(kRayOrderHistWords == kRayOrderBins + 32 + kScanBlocks && kRayOrderAlike == kRayOrderBins,
@@ -195,7 +197,7 @@ cudaError_t launch_ray_order(const float *o, const float *d, int64_t n, const fl
     k_ray_keys<true><<<grid, 256, 0, st>>>(o, d, n, key_grid(lo, hi, n), keys, hist, hist + kRayOrderAlike);
     k_scan_local<<<kScanBlocks, kScanThreads, 0, st>>>(hist, sums);
     k_scan_sums<<<1, kScanBlocks, 0, st>>>(sums);
-    k_ray_scatter<<<grid, 256, 0, st>>>(keys, n, hist, sums, perm);
+    k_ray_scatter<<<grid, 256, 0, st>>>(keys, n, hist, sums, perm, n_alike);
     return cudaGetLastError();
 }
 

@@ -201,7 +201,11 @@ def test_camera_rays_take_the_thread_form(form, order):
             for x, y in zip(got, want):
                 assert torch.equal(x, y[p])
     loss = ctx.opacity_loss(o, d, IDS)
-    assert ctx.last_form() == "thread"
+    gg = [torch.zeros(b.grid.shape, device="cuda") for b in sc.blocks]
+    gp = [[torch.zeros(p.shape, device="cuda") for p in b.planes] for b in sc.blocks]
+    ctx.render_backward(o[perm], d[perm], IDS, mlp, torch.zeros(n, 8, device="cuda"), torch.zeros(n, 3, device="cuda"),
+                        gg, gp, torch.zeros(499, device="cuda"))
+    assert ctx.last_form() == "thread"  # the opacity call's, whatever was ordered since
     again = ctx.opacity_loss(o[perm], d[perm], IDS)
     assert ctx.last_form() == "warp"
     assert abs(float(loss) - float(again)) <= 1e-5 * float(loss)
