@@ -484,8 +484,8 @@ cow_status cow_composite_over(cow_ctx *ctx, const float *o, const float *d, int6
                               float *out_aux, void *stream);
 
 /* cow_render_rays without early termination that also writes every block's
- * own transmittance prod (1 - alpha_i) over its occupied samples (Eq. 11),
- * -1 for a block without one: out_block_T is device float32 n_rays x n_ids,
+ * own transmittance prod (1 - alpha_i) over its occupied samples (Eq. 11), as
+ * exp(-sum sigma_i delta_i), -1 for a block without one: out_block_T is device float32 n_rays x n_ids,
  * row r, column k for ids[k].  cow_opacity_loss reads it instead of marching
  * each block a second time. */
 cow_status cow_render_rays_block_t(cow_ctx *ctx, const float *o, const float *d, int64_t n_rays, const int32_t *ids,
@@ -608,8 +608,9 @@ cow_status cow_update_features(cow_ctx *ctx, int32_t block, const float *grid, c
  *     block's opacity a = 1 - prod (1 - alpha_i) (Eq. 11), clamped to
  *     [1e-6, 1 - 1e-6]; the mean over rays of the sum over blocks.  No early
  *     termination.  block_T: NULL (every block is marched once for its
- *     opacity and once to scatter), or the out_block_T of a
- *     cow_render_rays_block_t call on the same rays and ids (one march).
+ *     opacity and once to scatter; large gradient calls keep the opacities in
+ *     n_rays x n_ids floats of context scratch in between), or the out_block_T
+ *     of a cow_render_rays_block_t call on the same rays and ids (one march).
  * Both add weight * loss to *loss (a device float; NULL: not computed) and
  * weight * d loss / d f0 into the FP32 gradient arrays, laid out as for
  * cow_render_backward (grad_grid / grad_planes both NULL: no gradient;

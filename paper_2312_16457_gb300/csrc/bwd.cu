@@ -21,9 +21,10 @@
 // K6's bound was the L2's rate of scattered reductions, 40 float4 a sample (one
 // ray per thread: 130 ms for 2^20 random rays over 2x2 blocks of 128^3 FP32,
 // 5.6e8 samples).  With a voxel's or texel's contributions added up before they
-// are reduced and the reductions in 64-byte groups it takes 65 ms, of which 35
-// are the reductions (timed without them); the rest is latency at 20 warps per SM
-// (issue slots 37 % busy, L1 data pipe 63 %, L2 53 %).
+// are reduced (25.5 float4 a sample, counted) and the reductions in 64-byte groups
+// it takes 65 ms, of which 35 are the reductions (timed without them); the rest
+// is latency at 20 warps per SM (100000 of the rays: issue slots 42 % busy, L1 data
+// pipe 73 %, L2 60 %).
 // The CTA's MLP weight gradient (499 sums over its 128 rays) goes to a
 // per-CTA scratch row; a second kernel adds the rows in a fixed order, so the
 // MLP gradient does not depend on scheduling.
@@ -583,9 +584,9 @@ __device__ __forceinline__ float opacity_term(const RegArgs &a, float a_raw) {
     return -(a.weight / (float)a.n_rays) * (al * logf(al) + (1.f - al) * log1pf(-al));
 }
 
-// Opacity, one ray per warp.  Bound by the L2's scattered reductions (65537 BF16
-// rays: a step of 8.4 ms, 12.1 ms with one ray per thread and 20 reductions a
-// sample).
+// Opacity, one ray per warp: 9.9 scalar reductions a sample instead of 20 (65537
+// BF16 rays: a training step of 8.4 ms, 12.1 ms with one ray per thread), then
+// bound by latency (issue slots 26 % busy, L1 data pipe 56 %, L2 42 %).
 template <int DT>
 __global__ void __launch_bounds__(kBwdThreads, COW_REG_MIN_BLOCKS) k_opacity(const __grid_constant__ RegArgs a,
                                                                           const __grid_constant__ RayRecs rr) {
